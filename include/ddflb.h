@@ -284,7 +284,8 @@ ddflb_status ddflb_reduce_noalloc(const ddflb_params* p, const void* dev_state,
  * 64x2, 32x4, 64x4, 32x8, 64x1) with each kernel variant (path 1: one node per
  * thread; path 2, 16-bit storage with even nx only: two adjacent nodes per
  * thread with aligned 4-byte pair accesses), and path 3 (four nodes per
- * thread, its own 128x1 block) once where it applies, over trial_steps with
+ * thread, its own 128x1 block) once where it applies, and path 0 once where it
+ * takes two steps per launch, over trial_steps with
  * CUDA events, and keeps the fastest.  Runs on zeroed populations, so it OVERWRITES the state and
  * resets the step counter: call it before ddflb_init.  Synchronises. */
 ddflb_status ddflb_autotune(ddflb_ctx* c, int32_t trial_steps, int32_t* block_x,
@@ -298,7 +299,9 @@ ddflb_status ddflb_set_block(ddflb_ctx* c, int32_t block_x, int32_t block_y);
  * 3 four adjacent nodes per thread with aligned 8-byte accesses (as 2, with
  * nx a multiple of 4; nodes next to a wall one by one; otherwise falls back to
  * 2, then 1);
- * 0 (default) = 3 for 16-bit storage (else 2 on a periodic lattice, else 1),
+ * 0 (default) = two steps per launch on large lattices (2^21 nodes or more,
+ * unforced, MRT or SRT scalar; single steps where a call or a residual check
+ * leaves one), else 3 for 16-bit storage (else 2 on a periodic lattice, else 1),
  * 1 for FP32.  All give bit-identical
  * results; which is faster depends on the shape, so the autotuner times them. */
 ddflb_status ddflb_set_path(ddflb_ctx* c, int32_t path);

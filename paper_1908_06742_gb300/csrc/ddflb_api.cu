@@ -194,7 +194,7 @@ struct ddflb_ctx {
   float* stage;
   int64_t step;
   int64_t snap_step;  // step at which uprev was last written (-1: none)
-  int path;           // step kernel: 0 default (16-bit storage: groups of 4 nodes, else
+  int path;           // step kernel: 0 default (large lattices: two steps per launch; 16-bit storage: groups of 4 nodes, else
                       // pairs on a periodic lattice, where eligible; else one node),
                       // 1 one node per thread, 2 paired nodes, 3 groups of 4 nodes
   float* stage_out;   // output staging area (host I/O)
@@ -204,6 +204,8 @@ struct ddflb_ctx {
   // (null: not built yet); graph_failed: capture unavailable, launch step by step
   cudaGraphExec_t step_graph[2];
   bool graph_failed;
+  int march_rows;     // rows per warp of the two-step kernel (0: one step per launch;
+                      // -1: not chosen yet)
   int32_t slab_y0;    // first global row of a y-slab context (0 for a whole lattice)
   int32_t global_ny;  // rows of the whole lattice
 };
@@ -252,12 +254,54 @@ cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void*
   return launch_step(c->L, fin, gin, fout, gout, c->status);
 }
 
+// Rows per warp of the two-step kernel (ddflb_march.cuh), or 0 where steps go
+// one per launch: the y-slab contexts, forced lattices and central-moment
+// scalar models (whose collisions have no packed form), an explicit path, and
+// lattices too small to fill the GPU with strips of enough rows.  Measured, two
+// steps per launch against the one-step kernels (us per step): FP32 1024^2 26
+// against 24.4, 2048^2 74 against 91.5; 16-bit 2048^2 cavity 59 against 65.5,
+// 1023 x 767 16.5 against 12.6.
+int choose_march_rows(const ddflb_ctx* c) {
+  const LbParams& P = c->L.P;
+  if (c->path != 0 || P.y0 != 0 || P.y1 != P.ny || c->L.force || P.smodel >= 2) return 0;
+  if ((int64_t)P.nx * P.ny < kMarchMinNodes) return 0;
+  // strips x chunks in waves of 15 warps an SM, plus most of a chunk at the end
+  // while the last ones finish (FP32 8192^2, rows 16 / 32 / 64 / 128: 878, 853,
+  // 870, 1023 us per step; 4096^2: 231, 237, 261, 325)
+  const double slots = 152 * 15;
+  const int strips = (P.nx + kMarchStrip - 1) / kMarchStrip;
+  double best = 1e300;
+  int rows = 16;
+  for (int r : {8, 12, 16, 24, 32, 48, 64}) {
+    const double n = (double)strips * ((P.ny + r - 1) / r);
+    const double cost = (n / slots + 1.0) * (r + 3);
+    if (cost < best) {
+      best = cost;
+      rows = r;
+    }
+  }
+  return rows;
+}
+
+// Two steps from buffer src into the other one.
+cudaError_t run_two(const ddflb_ctx* c, int src) {
+  const size_t gofs = c->lay.gofs;
+  const char* fi = (const char*)c->pops[src];
+  char* fo = (char*)c->pops[src ^ 1];
+  auto* launch = c->L.storage == 0   ? launch_march2_f32
+                 : c->L.storage == 1 ? launch_march2_f16
+                                     : launch_march2_bf16;
+  return launch(c->L, fi, fi + gofs, fo, fo + gofs, c->status, c->march_rows);
+}
+
 // Small lattices are launch-bound: runs of kGraphSteps steps between checks
 // replay one captured graph (an even count, so the buffer parity returns).
 // Only without a time-modulated force (whose factor changes every step).
 constexpr int kGraphSteps = 64;
 
+// Forget what was derived from the path and the force: graphs, rows per warp.
 void drop_graphs(ddflb_ctx* c) {
+  c->march_rows = -1;
   for (cudaGraphExec_t& g : c->step_graph)
     if (g) {
       cudaGraphExecDestroy(g);
@@ -280,7 +324,9 @@ cudaGraphExec_t step_graph(ddflb_ctx* c) {
   c->L.stream = cs;
   cudaGraph_t g = nullptr;
   bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-  for (int i = 0, cur = p; ok && i < kGraphSteps; ++i, cur ^= 1) {
+  for (int i = 0, cur = p; ok && c->march_rows > 0 && i < kGraphSteps; i += 2, cur ^= 1)
+    ok = run_two(c, cur) == cudaSuccess;
+  for (int i = 0, cur = p; ok && c->march_rows == 0 && i < kGraphSteps; ++i, cur ^= 1) {
     char* fo = (char*)c->pops[cur ^ 1];
     const size_t gofs = c->lay.gofs;
     ok = run_step(c, c->pops[cur], (const char*)c->pops[cur] + gofs, fo, fo + gofs) ==
@@ -313,6 +359,11 @@ ddflb_status reset_status(ddflb_ctx* c) {
 }
 
 const void* gptr(const ddflb_ctx* c, int buf) { return (const char*)c->pops[buf] + c->lay.gofs; }
+
+ddflb_status timed_out(const ddflb_ctx* c) {
+  return fail(DDFLB_ETIMEOUT, "a bulk copy of the step kernel did not arrive (step %lld)",
+              (long long)c->step);
+}
 
 ddflb_status check_launch(cudaError_t e, const char* where) {
   return e == cudaSuccess ? DDFLB_OK : cuda_fail(e, where);
@@ -409,6 +460,7 @@ ddflb_status create_ctx(const ddflb_params* p, int glo, int ghi, int32_t y0, int
   c->L.stream = (cudaStream_t)stream;
   c->step = 0;
   c->snap_step = -1;
+  c->march_rows = -1;
   ddflb_status st = reset_status(c);
   if (st != DDFLB_OK) {
     delete c;
@@ -519,6 +571,7 @@ ddflb_status ddflb_step(ddflb_ctx* c, int64_t n) {
                               "refreshed between steps");
   Range range("ddflb_step");
   const int K = c->p.check_every;
+  if (c->march_rows < 0) c->march_rows = choose_march_rows(c);
   while (n > 0) {
     if (c->p.force_omega == 0.0 && !c->graph_failed) {
       // whole graphs up to the next check step (checks run after it, as below)
@@ -538,6 +591,16 @@ ddflb_status ddflb_step(ddflb_ctx* c, int64_t n) {
         if (s != DDFLB_OK) return s;
         continue;
       }
+    }
+    if (n > 1 && c->march_rows > 0 && (K == 0 || K - c->step % K >= 2)) {
+      cudaError_t e = run_two(c, c->cur);
+      if (e != cudaSuccess) return cuda_fail(e, "step");
+      c->cur ^= 1;
+      c->step += 2;
+      n -= 2;
+      ddflb_status s = checks_at(c);
+      if (s != DDFLB_OK) return s;
+      continue;
     }
     --n;
     const int src = c->cur, dst = c->cur ^ 1;
@@ -656,6 +719,7 @@ ddflb_status ddflb_stats(ddflb_ctx* c, double* mass, double* scalar, double* res
   if (scalar) *scalar = cells * c->p.phi0 + h.scalar_dev;
   if (residual) *residual = h.has_residual ? h.residual / c->p.check_every : NAN;
   if (step) *step = c->step;
+  if (h.timeout) return timed_out(c);
   if (h.diverged) return fail(DDFLB_EDIVERGED, "non-finite mass/scalar sum by step %lld",
                               (long long)c->step);
   return DDFLB_OK;
@@ -687,6 +751,7 @@ ddflb_status ddflb_run_to_tolerance(ddflb_ctx* c, double tol, int64_t max_steps,
     cudaError_t e = cudaMemcpyAsync(&h, c->status, sizeof h, cudaMemcpyDeviceToHost, c->L.stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->L.stream);
     if (e != cudaSuccess) return cuda_fail(e, "run_to_tolerance");
+    if (h.timeout) return timed_out(c);
     if (h.diverged)
       return fail(DDFLB_EDIVERGED, "non-finite mass/scalar sum by step %lld", (long long)c->step);
     if (!h.has_residual) continue;  // the first check only takes the snapshot
@@ -788,6 +853,26 @@ ddflb_status ddflb_autotune(ddflb_ctx* c, int32_t trial_steps, int32_t* block_x,
         bestb = c->L.block;
         bestp = pth;
       }
+    }
+  }
+  // the automatic path, where it takes two steps per launch (at the default block)
+  c->path = 0;
+  c->march_rows = choose_march_rows(c);
+  if (c->march_rows > 0 && e == cudaSuccess) {
+    const int pairs = (trial_steps + 1) / 2;
+    for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
+      if (rep == 1) e = cudaEventRecord(e0, s);
+      for (int i = 0; i < pairs && e == cudaSuccess; ++i) e = run_two(c, i & 1);
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(e1, s);
+    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    float ms = 0.f;
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    ms *= (float)trial_steps / (2 * pairs);
+    if (e == cudaSuccess && ms < best) {
+      best = ms;
+      bestb = dim3(128, 1, 1);
+      bestp = 0;
     }
   }
   cudaEventDestroy(e0);
@@ -902,6 +987,7 @@ ddflb_status ddflb_sums(ddflb_ctx* c, int32_t mode, double* out) {
   out[1] = h.scalar_dev;
   out[2] = h.u2;
   out[3] = (mode & 1) ? h.du2 : NAN;
+  if (h.timeout) return timed_out(c);
   if (h.diverged) return fail(DDFLB_EDIVERGED, "non-finite sum by step %lld", (long long)c->step);
   return DDFLB_OK;
 }

@@ -64,7 +64,8 @@ struct DevStatus {
   double residual;    // sqrt(du2 / u2) of the last check
   int32_t diverged;   // set once a sum is non-finite
   int32_t has_residual;
-  int64_t pad;
+  int32_t timeout;    // a bulk copy of the two-step kernel did not arrive in time
+  int32_t pad;
 };
 
 // ------------------------------------------------------------ storage codec
@@ -81,6 +82,8 @@ template <> struct Codec<float> {
   template <bool COH = false>
   static __device__ __forceinline__ float load(const float* p, float) { return ld_pop<COH>(p); }
   static __device__ __forceinline__ void store(float* p, float v, float) { __stcs(p, v); }
+  // get: the same conversion from shared memory
+  static __device__ __forceinline__ float get(const float* p, float) { return *p; }
 };
 template <> struct Codec<__half> {
   template <bool COH = false>
@@ -90,6 +93,9 @@ template <> struct Codec<__half> {
   static __device__ __forceinline__ void store(__half* p, float v, float s) {
     __stcs(reinterpret_cast<unsigned short*>(p), __half_as_ushort(__float2half_rn(v * s)));
   }
+  static __device__ __forceinline__ float get(const __half* p, float inv) {
+    return __half2float(*p) * inv;
+  }
 };
 template <> struct Codec<__nv_bfloat16> {
   template <bool COH = false>
@@ -98,6 +104,9 @@ template <> struct Codec<__nv_bfloat16> {
   }
   static __device__ __forceinline__ void store(__nv_bfloat16* p, float v, float s) {
     __stcs(reinterpret_cast<unsigned short*>(p), __bfloat16_as_ushort(__float2bfloat16_rn(v * s)));
+  }
+  static __device__ __forceinline__ float get(const __nv_bfloat16* p, float inv) {
+    return __bfloat162float(*p) * inv;
   }
 };
 

@@ -9,6 +9,8 @@
 
 namespace ddflb {
 
+constexpr int kMarchStrip = 60;  // columns of a strip of the two-step kernel
+constexpr int64_t kMarchMinNodes = (int64_t)1 << 21;  // smallest lattice it is used for
 constexpr int kReduceThreads = 256;
 constexpr int kReduceBlocks = 608;  // 4 per SM on a 152-SM GB300; fixed for deterministic sums
 
@@ -53,6 +55,13 @@ cudaError_t launch_halo_local(const HaloSlabs& H, int storage, cudaStream_t stre
 
 cudaError_t launch_step(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                         const DevStatus* st);
+// two time steps in one launch (ddflb_march.cuh); rows: lattice rows per CTA
+cudaError_t launch_march2_f32(const Launch& L, const void* fin, const void* gin, void* fout,
+                              void* gout, DevStatus* st, int rows);
+cudaError_t launch_march2_f16(const Launch& L, const void* fin, const void* gin, void* fout,
+                              void* gout, DevStatus* st, int rows);
+cudaError_t launch_march2_bf16(const Launch& L, const void* fin, const void* gin, void* fout,
+                               void* gout, DevStatus* st, int rows);
 cudaError_t launch_fields(const Launch& L, const void* fin, const void* gin, const FieldPtrs& out);
 cudaError_t launch_pops(const Launch& L, const void* fin, const void* gin, float* f, float* g);
 cudaError_t launch_init(const Launch& L, const InitPtrs& in, void* fout, void* gout);
