@@ -206,6 +206,7 @@ struct ddflb_ctx {
   bool graph_failed;
   int march_rows;     // rows per warp of the two-step kernel (0: one step per launch;
                       // -1: not chosen yet)
+  int tile;           // tile shape of the multi-step kernel (-1: not used)
   int32_t slab_y0;    // first global row of a y-slab context (0 for a whole lattice)
   int32_t global_ny;  // rows of the whole lattice
 };
@@ -294,6 +295,34 @@ cudaError_t run_two(const ddflb_ctx* c, int src) {
   return launch(c->L, fi, fi + gofs, fo, fo + gofs, c->status, c->march_rows);
 }
 
+// Tile shape of the multi-step kernel (ddflb_tile.cuh), or -1 where it is not
+// used: the smallest shape whose tiles are no more than the SMs, so that every
+// launch is one wave (288 tiles of 8 x 4 on a 96^2 cavity 1.19 us per step, 144
+// of 8 x 8 1.12).  Beyond 152 of the largest tiles single steps are faster
+// (384^2: 4.1 us per step, two or four steps per launch 4.3).
+int choose_tile(const ddflb_ctx* c) {
+  const LbParams& P = c->L.P;
+  if (c->path != 0 || P.y0 != 0 || P.y1 != P.ny || c->p.force_omega != 0.0 || P.smodel >= 2)
+    return -1;
+  if (P.nx < kTileSteps || P.ny < kTileSteps) return -1;  // (a region wraps once at most)
+  for (int k = 0; k < kTileShapes; ++k) {
+    const int tx = kTileShape[k][0], ty = kTileShape[k][1];
+    if ((int64_t)((P.nx + tx - 1) / tx) * ((P.ny + ty - 1) / ty) <= 152) return k;
+  }
+  return -1;
+}
+
+// kTileSteps steps from buffer src into the other one.
+cudaError_t run_tile(const ddflb_ctx* c, int src) {
+  const size_t gofs = c->lay.gofs;
+  const char* fi = (const char*)c->pops[src];
+  char* fo = (char*)c->pops[src ^ 1];
+  auto* launch = c->L.storage == 0   ? launch_tile_f32
+                 : c->L.storage == 1 ? launch_tile_f16
+                                     : launch_tile_bf16;
+  return launch(c->L, fi, fi + gofs, fo, fo + gofs, c->status, c->tile);
+}
+
 // Small lattices are launch-bound: runs of kGraphSteps steps between checks
 // replay one captured graph (an even count, so the buffer parity returns).
 // Only without a time-modulated force (whose factor changes every step).
@@ -326,7 +355,10 @@ cudaGraphExec_t step_graph(ddflb_ctx* c) {
   bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
   for (int i = 0, cur = p; ok && c->march_rows > 0 && i < kGraphSteps; i += 2, cur ^= 1)
     ok = run_two(c, cur) == cudaSuccess;
-  for (int i = 0, cur = p; ok && c->march_rows == 0 && i < kGraphSteps; ++i, cur ^= 1) {
+  for (int i = 0, cur = p; ok && c->tile >= 0 && i < kGraphSteps; i += kTileSteps, cur ^= 1)
+    ok = run_tile(c, cur) == cudaSuccess;
+  const bool single = c->march_rows == 0 && c->tile < 0;
+  for (int i = 0, cur = p; ok && single && i < kGraphSteps; ++i, cur ^= 1) {
     char* fo = (char*)c->pops[cur ^ 1];
     const size_t gofs = c->lay.gofs;
     ok = run_step(c, c->pops[cur], (const char*)c->pops[cur] + gofs, fo, fo + gofs) ==
@@ -460,7 +492,7 @@ ddflb_status create_ctx(const ddflb_params* p, int glo, int ghi, int32_t y0, int
   c->L.stream = (cudaStream_t)stream;
   c->step = 0;
   c->snap_step = -1;
-  c->march_rows = -1;
+  c->march_rows = c->tile = -1;
   ddflb_status st = reset_status(c);
   if (st != DDFLB_OK) {
     delete c;
@@ -571,7 +603,10 @@ ddflb_status ddflb_step(ddflb_ctx* c, int64_t n) {
                               "refreshed between steps");
   Range range("ddflb_step");
   const int K = c->p.check_every;
-  if (c->march_rows < 0) c->march_rows = choose_march_rows(c);
+  if (c->march_rows < 0) {
+    c->march_rows = choose_march_rows(c);
+    c->tile = choose_tile(c);
+  }
   while (n > 0) {
     if (c->p.force_omega == 0.0 && !c->graph_failed) {
       // whole graphs up to the next check step (checks run after it, as below)
@@ -598,6 +633,17 @@ ddflb_status ddflb_step(ddflb_ctx* c, int64_t n) {
       c->cur ^= 1;
       c->step += 2;
       n -= 2;
+      ddflb_status s = checks_at(c);
+      if (s != DDFLB_OK) return s;
+      continue;
+    }
+    constexpr int T = kTileSteps;
+    if (c->tile >= 0 && n >= T && (K == 0 || K - c->step % K >= T)) {
+      cudaError_t e = run_tile(c, c->cur);
+      if (e != cudaSuccess) return cuda_fail(e, "step");
+      c->cur ^= 1;
+      c->step += T;
+      n -= T;
       ddflb_status s = checks_at(c);
       if (s != DDFLB_OK) return s;
       continue;

@@ -82,8 +82,9 @@ template <> struct Codec<float> {
   template <bool COH = false>
   static __device__ __forceinline__ float load(const float* p, float) { return ld_pop<COH>(p); }
   static __device__ __forceinline__ void store(float* p, float v, float) { __stcs(p, v); }
-  // get: the same conversion from shared memory
+  // get / put: the same conversions without cache hints (shared memory)
   static __device__ __forceinline__ float get(const float* p, float) { return *p; }
+  static __device__ __forceinline__ void put(float* p, float v, float) { *p = v; }
 };
 template <> struct Codec<__half> {
   template <bool COH = false>
@@ -96,6 +97,9 @@ template <> struct Codec<__half> {
   static __device__ __forceinline__ float get(const __half* p, float inv) {
     return __half2float(*p) * inv;
   }
+  static __device__ __forceinline__ void put(__half* p, float v, float s) {
+    *p = __float2half_rn(v * s);
+  }
 };
 template <> struct Codec<__nv_bfloat16> {
   template <bool COH = false>
@@ -107,6 +111,9 @@ template <> struct Codec<__nv_bfloat16> {
   }
   static __device__ __forceinline__ float get(const __nv_bfloat16* p, float inv) {
     return __bfloat162float(*p) * inv;
+  }
+  static __device__ __forceinline__ void put(__nv_bfloat16* p, float v, float s) {
+    *p = __float2bfloat16_rn(v * s);
   }
 };
 

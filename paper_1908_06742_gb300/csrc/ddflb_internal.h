@@ -62,6 +62,16 @@ cudaError_t launch_march2_f16(const Launch& L, const void* fin, const void* gin,
                               void* gout, DevStatus* st, int rows);
 cudaError_t launch_march2_bf16(const Launch& L, const void* fin, const void* gin, void* fout,
                                void* gout, DevStatus* st, int rows);
+// several time steps per launch on small lattices (ddflb_tile.cuh): the tile
+// shapes it is built for, smallest first
+constexpr int kTileSteps = 4, kTileShapes = 5;
+constexpr int kTileShape[kTileShapes][2] = {{8, 4}, {8, 8}, {16, 8}, {16, 16}, {32, 14}};
+cudaError_t launch_tile_f32(const Launch& L, const void* fin, const void* gin, void* fout,
+                            void* gout, const DevStatus* st, int shape);
+cudaError_t launch_tile_f16(const Launch& L, const void* fin, const void* gin, void* fout,
+                            void* gout, const DevStatus* st, int shape);
+cudaError_t launch_tile_bf16(const Launch& L, const void* fin, const void* gin, void* fout,
+                             void* gout, const DevStatus* st, int shape);
 cudaError_t launch_fields(const Launch& L, const void* fin, const void* gin, const FieldPtrs& out);
 cudaError_t launch_pops(const Launch& L, const void* fin, const void* gin, float* f, float* g);
 cudaError_t launch_init(const Launch& L, const InitPtrs& in, void* fout, void* gout);
