@@ -521,6 +521,22 @@ ddflb_status ddflb_nn_conv3x3(const void* X, int32_t B, int32_t H, int32_t W, in
  * chunk), elsewhere one box per tap; 1 = one box per tap everywhere.  Same results bit for bit
  * (the K order is the im2col order in both). */
 ddflb_status ddflb_nn_set_conv_path(int32_t path);
+/* The same convolution for C = 16, 32 or 64 channels and any image size whose
+ * tile fits shared memory (W a multiple of 128, or up to 250 and more where C
+ * is small; else EINVAL): each tile of 128 positions is copied once with its
+ * halo and read by all nine taps.  Bit-identical to im2col + ddflb_nn_gemm.
+ * ddflb_nn_conv3x3 takes this form for C = 64 on path 0. */
+ddflb_status ddflb_nn_conv3x3_narrow(const void* X, int32_t B, int32_t H, int32_t W, int32_t C,
+                                     int32_t cs, const void* Wt, int32_t N, float* Cf, int32_t ldc,
+                                     void* Cb, int32_t ldcb, const float* bias, int32_t act,
+                                     int32_t accumulate, void* stream);
+/* Input gradient dX [B H W][ldc] FP32 of Y = conv3x3(X, Wt) from dY = G BF16
+ * NHWC with Co = 16, 32 or 64 channels (Wt BF16 [Co][9 Ci]): the nine taps'
+ * products rounded one by one and added in tap order, bit-identical to the GEMM
+ * with the transposed weights followed by ddflb_nn_col2im. */
+ddflb_status ddflb_nn_conv3x3_dgrad(const void* G, int32_t B, int32_t H, int32_t W, int32_t Co,
+                                    int32_t cs, const void* Wt, int32_t Ci, float* dX, int32_t ldc,
+                                    void* stream);
 /* Weights of the adjoint convolution: Wf[ci][t][co] = Wt[co][8 - t][ci]
  * (BF16, Wt [Co][9][Ci] -> Wf [Ci][9][Co]), so that dX = conv3x3(dY, Wf)
  * with C = Co and N = Ci is the input gradient of Y = conv3x3(X, Wt). */

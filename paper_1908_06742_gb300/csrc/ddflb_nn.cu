@@ -906,6 +906,8 @@ __global__ void __launch_bounds__(tcp::THREADS, 1) k_gemm_tcp(
   }
 }
 
+#include "ddflb_nn_narrow.cuh"
+
 // split-K: C = sum over slices z (fixed order) of partial[z]; then bias, act
 __global__ void k_splitk_reduce(const float* __restrict__ partial, int splits, int M, int N,
                                 float* __restrict__ Cf, int ldc, const float* __restrict__ bias,
@@ -1566,6 +1568,71 @@ ddflb_status ddflb_nn_conv3x3(const void* X, int32_t B, int32_t H, int32_t W, in
   if (128 % bw || (W >= 128 && W % 128) || H % bh || bw * bh * bb != 128 || B % bb ||
       ((int64_t)B * H * W) % 128 || (int64_t)B * H * W > INT32_MAX)
     return bad("conv3x3: 128-pixel tiles need W a divisor of 128 or a multiple of it, and whole "
+// Geometry of a narrow convolution with mt units of 128 positions per tile;
+// false where it does not apply.
+bool narrow_args(narrow::Args* a, const void* X, int B, int H, int W, int C, int cs,
+                 const void* Wt, int bn, int mt, const GemmArgs& g) {
+  *a = narrow::Args{};
+  a->X = (const bf16*)X;
+  a->B = B;
+  a->H = H;
+  a->W = W;
+  a->cs = cs;
+  a->Wt = (const bf16*)Wt;
+  a->segment = W % 128 == 0;
+  a->pitch = a->segment ? 130 : W + 2;
+  a->inv_pitch = 0xffffffffu / (uint32_t)a->pitch + 1u;
+  a->npos = a->segment ? (mt + 2) * 130 : mt * 128 + 2 * a->pitch + 2;
+  a->unit_step = a->segment ? 130 : 128;
+  const int64_t per = a->segment ? (int64_t)((H + mt - 1) / mt) * (W / 128)
+                                 : ((int64_t)H * a->pitch + 128 * mt - 1) / (128 * mt);
+  if (per * B > INT32_MAX / 512 || ((int64_t)H + 8) * a->pitch * a->pitch >= (int64_t)1 << 32)
+    return false;  // (and positions / pitch by one multiplication)
+  a->per_img = (int)per;
+  a->tiles = (int)(per * B);
+  a->ntn = (g.N + bn - 1) / bn;
+  a->g = g;
+  const int64_t weights = 9 * (C / 8) * (int64_t)bn * 16, buf = (C / 8) * (int64_t)a->npos * 16;
+  for (a->nbuf = 4; a->nbuf >= 2; --a->nbuf)
+    if (weights + a->nbuf * buf <= tcp::SMEM_MAX) return a->ntn <= sm_count();
+  return false;
+}
+
+template <int CH, int BN, bool SEP, int MT>
+ddflb_status narrow_run(const narrow::Args& a, cudaStream_t s) {
+  auto* kernel = narrow::k_conv_narrow<CH, BN, SEP, MT>;
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tcp::SMEM_MAX);
+  if (attr != cudaSuccess) return bad("narrow convolution: shared memory attribute");
+  const int smem = 9 * CH * BN * 16 + a.nbuf * CH * a.npos * 16;
+  const int per = sm_count() / a.ntn;
+  kernel<<<(a.tiles < per ? a.tiles : per) * a.ntn, narrow::THREADS, smem, s>>>(a);
+  return launched("narrow convolution");
+}
+
+// Two units per tile where every SM still gets one (64^2, 64 -> 64, 16 images:
+// 16.5 us, one unit per tile 18.5), else one unit.  `refused`: whether the shape
+// does not fit at all.
+template <int CH, int BN, bool SEP>
+ddflb_status narrow_go(const void* X, int B, int H, int W, int cs, const void* Wt,
+                       const GemmArgs& g, cudaStream_t s, bool* refused) {
+  narrow::Args a;
+  *refused = false;
+  if (narrow_args(&a, X, B, H, W, 8 * CH, cs, Wt, BN, 2, g) && 
+      a.tiles >= sm_count() / a.ntn)
+    return narrow_run<CH, BN, SEP, 2>(a, s);
+  if (narrow_args(&a, X, B, H, W, 8 * CH, cs, Wt, BN, 1, g)) return narrow_run<CH, BN, SEP, 1>(a, s);
+  *refused = true;
+  return bad("convolution: rows too wide for a tile in shared memory");
+}
+
+template <int CH>
+ddflb_status narrow_fwd(const void* X, int B, int H, int W, int cs, const void* Wt,
+                        const GemmArgs& g, cudaStream_t s, bool* refused) {
+  return g.N <= 32 ? narrow_go<CH, 32, false>(X, B, H, W, cs, Wt, g, s, refused)
+                   : narrow_go<CH, 64, false>(X, B, H, W, cs, Wt, g, s, refused);
+}
+
                "boxes of rows and images");
   GemmArgs g{};
   g.A = (const bf16*)X;
@@ -1719,12 +1786,66 @@ ddflb_status ddflb_nn_mse(const float* pred, const float* target, int64_t n, flo
   return launched("mse");
 }
 
+  if (C == 64 && g_conv_path == 0) {
+    bool refused;
+    const ddflb_status st = narrow_fwd<8>(X, B, H, W, cs, Wt, g, s, &refused);
+    if (!refused) return st;
+  }
 ddflb_status ddflb_nn_adam(float* w, const float* g, float* m, float* v, void* wb, int64_t n,
                            float lr, float beta1, float beta2, float eps, int64_t t, float wd,
                            void* stream) {
   if (!w || !g || !m || !v || n <= 0 || t < 1) return bad("adam: bad args");
   const float c1 = 1.f - powf(beta1, (float)t), c2 = 1.f - powf(beta2, (float)t);
   k_adam<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(w, g, m, v, (bf16*)wb, n, lr, beta1,
+ddflb_status ddflb_nn_conv3x3_narrow(const void* X, int32_t B, int32_t H, int32_t W, int32_t C,
+                                     int32_t cs, const void* Wt, int32_t N, float* Cf, int32_t ldc,
+                                     void* Cb, int32_t ldcb, const float* bias, int32_t act,
+                                     int32_t accumulate, void* stream) {
+  if (!X || !Wt || B <= 0 || H <= 0 || W <= 0 || N <= 0 || (!Cf && !Cb))
+    return bad("conv3x3_narrow: bad arguments");
+  if ((C != 16 && C != 32 && C != 64) || cs < C || cs % 8 || ((uintptr_t)X % 16) ||
+      ((uintptr_t)Wt % 16))
+    return bad("conv3x3_narrow: C must be 16, 32 or 64, cs a multiple of 8 (>= C), X and Wt "
+               "16-byte aligned");
+  if ((Cf && ldc < N) || (Cb && ldcb < N)) return bad("conv3x3_narrow: leading dims");
+  if (act < 0 || act > 1) return bad("conv3x3_narrow: act must be 0 (none) or 1 (leaky ReLU)");
+  GemmArgs g{};
+  g.N = N;
+  g.Cf = Cf;
+  g.Cb = (bf16*)Cb;
+  g.ldc = ldc;
+  g.ldcb = ldcb;
+  g.bias = bias;
+  g.act = act;
+  g.accumulate = accumulate;
+  cudaStream_t s = (cudaStream_t)stream;
+  if ((int64_t)B * H * W > INT32_MAX) return bad("conv3x3_narrow: too many pixels");
+  bool refused;
+  return C == 16   ? narrow_fwd<2>(X, B, H, W, cs, Wt, g, s, &refused)
+         : C == 32 ? narrow_fwd<4>(X, B, H, W, cs, Wt, g, s, &refused)
+                   : narrow_fwd<8>(X, B, H, W, cs, Wt, g, s, &refused);
+}
+
+ddflb_status ddflb_nn_conv3x3_dgrad(const void* G, int32_t B, int32_t H, int32_t W, int32_t Co,
+                                    int32_t cs, const void* Wt, int32_t Ci, float* dX, int32_t ldc,
+                                    void* stream) {
+  if (!G || !Wt || !dX || B <= 0 || H <= 0 || W <= 0 || Ci <= 0)
+    return bad("conv3x3_dgrad: bad arguments");
+  if ((Co != 16 && Co != 32 && Co != 64) || cs < Co || cs % 8 || ((uintptr_t)G % 16) || ldc < Ci)
+    return bad("conv3x3_dgrad: Co must be 16, 32 or 64, cs a multiple of 8 (>= Co), G 16-byte "
+               "aligned, ldc >= Ci");
+  GemmArgs g{};
+  g.N = Ci;
+  g.Cf = dX;
+  g.ldc = ldc;
+  cudaStream_t s = (cudaStream_t)stream;
+  if ((int64_t)B * H * W > INT32_MAX) return bad("conv3x3_dgrad: too many pixels");
+  bool refused;
+  return Co == 16   ? narrow_go<2, 32, true>(G, B, H, W, cs, Wt, g, s, &refused)
+         : Co == 32 ? narrow_go<4, 32, true>(G, B, H, W, cs, Wt, g, s, &refused)
+                    : narrow_go<8, 32, true>(G, B, H, W, cs, Wt, g, s, &refused);
+}
+
                                                          beta2, eps, c1, c2, wd);
   return launched("adam");
 }

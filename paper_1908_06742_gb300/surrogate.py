@@ -64,8 +64,8 @@ class UNet:
         import torch
         assert H % 8 == 0 and W % 8 == 0
         self.torch = torch
-        # 3x3 convolutions with >= 64 input channels as implicit GEMMs (no
-        # patch matrix); the others through im2col + GEMM
+        # 3x3 convolutions as implicit GEMMs (no patch matrix) where the kernels
+        # take the layer; else through im2col + GEMM
         self.implicit = implicit
         self.c, self.B, self.H, self.W = c, batch, H, W
         self.dev = torch.device(device)
@@ -170,6 +170,15 @@ class UNet:
         return (128 % bw == 0 and (W < 128 or W % 128 == 0) and H % bh == 0
                 and bw * bh * bb == 128 and self.B % bb == 0)
 
+    def _narrow_ok(self, C, W, bn):
+        """ddflb_nn_conv3x3_narrow / _dgrad take this layer: 16, 32 or 64 input
+        channels, two tiles (with halo) and the weights of bn outputs in shared
+        memory."""
+        if not self.implicit or C not in (16, 32, 64):
+            return False
+        npos = 390 if W % 128 == 0 else 128 + 2 * (W + 2) + 2
+        return 2 * C * (9 * bn + 2 * npos) <= 226 * 1024
+
     def _conv_fwd(self, name, lv, vin, vout):
         p = self.p[name]
         H, W = self.L[lv]
@@ -180,6 +189,11 @@ class UNet:
             _ck(self.lib.ddflb_nn_conv3x3(vin.ptr, self.B, H, W, ci, vin.cs, p["wb"].data_ptr(),
                                           co, None, 0, vout.ptr, vout.cs, p["b"].data_ptr(),
                                           LEAKY, 0, self.s))
+            return
+        if self._narrow_ok(ci, W, 32 if co <= 32 else 64):
+            _ck(self.lib.ddflb_nn_conv3x3_narrow(vin.ptr, self.B, H, W, ci, vin.cs,
+                                                 p["wb"].data_ptr(), co, None, 0, vout.ptr,
+                                                 vout.cs, p["b"].data_ptr(), LEAKY, 0, self.s))
             return
         _ck(self.lib.ddflb_nn_im2col(vin.ptr, self.B, H, W, ci, vin.cs, self.col.data_ptr(), 0,
                                      self.s))
@@ -209,6 +223,11 @@ class UNet:
                                                self.s))
             _ck(self.lib.ddflb_nn_conv3x3(gbf, self.B, H, W, co, co, p["wT"].data_ptr(), ci,
                                           gin.ptr, gin.cs, None, 0, None, 0, 0, self.s))
+            return
+        if self._narrow_ok(co, W, 32):
+            # dX tap by tap, without the patch columns of the gradient
+            _ck(self.lib.ddflb_nn_conv3x3_dgrad(gbf, self.B, H, W, co, co, p["wb"].data_ptr(), ci,
+                                                gin.ptr, gin.cs, self.s))
             return
         # dX = col2im(g . W)
         _ck(self.lib.ddflb_nn_transpose(p["wb"].data_ptr(), co, 9 * ci, 9 * ci,
