@@ -1142,6 +1142,85 @@ __global__ void k_upsample_bwd(const float* __restrict__ dY, int B, int H, int W
   }
 }
 
+// Vector forms of the four above, one thread per coarse pixel and chunk of
+// channels (8 BF16 or 4 FP32, 16 bytes; C and the strides multiples of that,
+// buffers 16-byte aligned): a quarter of the index arithmetic and 16-byte
+// accesses.  The sums keep their order.  B = 16, 256^2, 32 channels: pool
+// 57 -> 15 us, upsample (128^2, 64 channels) 171 -> 26 us.
+__global__ void k_pool_v8(const bf16* __restrict__ X, uint32_t total, int H, int W, int C8,
+                          int csx, bf16* __restrict__ Y, int csy) {
+  const uint32_t Ho = H / 2, Wo = W / 2;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const uint32_t p = i / C8, c = (i - p * C8) * 8;
+    const uint32_t t = p / Wo, w = p - t * Wo, b = t / Ho, h = t - b * Ho;
+    const bf16* x = X + (((size_t)b * H + 2 * h) * W + 2 * w) * csx + c;
+    uint4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      v[k] = __ldg(reinterpret_cast<const uint4*>(x + ((size_t)(k >> 1) * W + (k & 1)) * csx));
+    __align__(16) bf16 o[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      float s = 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s += __bfloat162float(reinterpret_cast<const bf16*>(&v[k])[e]);
+      o[e] = __float2bfloat16_rn(0.25f * s);
+    }
+    *reinterpret_cast<uint4*>(Y + (size_t)p * csy + c) = *reinterpret_cast<const uint4*>(o);
+  }
+}
+
+__global__ void k_upsample_v8(const bf16* __restrict__ X, uint32_t total, int H, int W, int C8,
+                              int csx, bf16* __restrict__ Y, int csy) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const uint32_t p = i / C8, c = (i - p * C8) * 8;
+    const uint32_t t = p / W, w = p - t * W;  // t = b H + h
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(X + (size_t)p * csx + c));
+    bf16* y = Y + ((size_t)t * 4 * W + 2 * w) * csy + c;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      *reinterpret_cast<uint4*>(y + ((size_t)(k >> 1) * 2 * W + (k & 1)) * csy) = v;
+  }
+}
+
+__global__ void k_pool_bwd_v4(const float* __restrict__ dY, uint32_t total, int W, int C4, int csy,
+                              float* __restrict__ dX, int csx, int accumulate) {
+  const uint32_t Wo = W / 2;  // total counts coarse pixels x chunks
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const uint32_t p = i / C4, c = (i - p * C4) * 4;
+    const uint32_t t = p / Wo, w = p - t * Wo;
+    const float4 q = __ldg(reinterpret_cast<const float4*>(dY + (size_t)p * csy + c));
+    float* x = dX + ((size_t)t * 2 * W + 2 * w) * csx + c;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float4* d = reinterpret_cast<float4*>(x + ((size_t)(k >> 1) * W + (k & 1)) * csx);
+      float4 o = make_float4(0.25f * q.x, 0.25f * q.y, 0.25f * q.z, 0.25f * q.w);
+      if (accumulate) {
+        const float4 a = *d;
+        o = make_float4(a.x + o.x, a.y + o.y, a.z + o.z, a.w + o.w);
+      }
+      *d = o;
+    }
+  }
+}
+
+__global__ void k_upsample_bwd_v4(const float* __restrict__ dY, uint32_t total, int W, int C4,
+                                  int csy, float* __restrict__ dX, int csx) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const uint32_t p = i / C4, c = (i - p * C4) * 4;
+    const uint32_t t = p / W, w = p - t * W;
+    const float* y = dY + ((size_t)t * 4 * W + 2 * w) * csy + c;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 v =
+          __ldg(reinterpret_cast<const float4*>(y + ((size_t)(k >> 1) * 2 * W + (k & 1)) * csy));
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    *reinterpret_cast<float4*>(dX + (size_t)p * csx + c) = s;
+  }
+}
+
 // gradient through the activation: g *= f'(z), with f' read from the output y
 // (leaky ReLU: 1 where y > 0, else the slope); writes FP32 and a BF16 copy
 __global__ void k_act_bwd(float* __restrict__ g, const bf16* __restrict__ y, int64_t rows, int C,
@@ -1155,6 +1234,30 @@ __global__ void k_act_bwd(float* __restrict__ g, const bf16* __restrict__ y, int
     if (act == 1 && !(__bfloat162float(y[r * csy + c]) > 0.f)) v *= 0.02f;
     g[r * csg + c] = v;
     if (gb) gb[r * csb + c] = __float2bfloat16_rn(v);
+  }
+}
+
+// four channels per thread (C and the strides multiples of 4, 16-byte aligned)
+__global__ void k_act_bwd_v4(float* __restrict__ g, const bf16* __restrict__ y, uint32_t total,
+                             int C4, int csg, int csy, int act, bf16* __restrict__ gb, int csb) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const uint32_t r = i / C4, c = (i - r * C4) * 4;
+    float4* gp = reinterpret_cast<float4*>(g + (size_t)r * csg + c);
+    float4 v = *gp;
+    if (act == 1) {
+      const uint2 yw = __ldg(reinterpret_cast<const uint2*>(y + (size_t)r * csy + c));
+      const bf16* e = reinterpret_cast<const bf16*>(&yw);
+      if (!(__bfloat162float(e[0]) > 0.f)) v.x *= 0.02f;
+      if (!(__bfloat162float(e[1]) > 0.f)) v.y *= 0.02f;
+      if (!(__bfloat162float(e[2]) > 0.f)) v.z *= 0.02f;
+      if (!(__bfloat162float(e[3]) > 0.f)) v.w *= 0.02f;
+      *gp = v;
+    }
+    if (gb) {
+      __align__(8) bf16 o[4] = {__float2bfloat16_rn(v.x), __float2bfloat16_rn(v.y),
+                                __float2bfloat16_rn(v.z), __float2bfloat16_rn(v.w)};
+      *reinterpret_cast<uint2*>(gb + (size_t)r * csb + c) = *reinterpret_cast<const uint2*>(o);
+    }
   }
 }
 
@@ -1173,8 +1276,19 @@ __global__ void __launch_bounds__(256) k_bias_grad_part(const float* __restrict_
   const int64_t per = (rows + gridDim.y - 1) / gridDim.y;
   const int64_t r0 = blockIdx.y * per, r1 = r0 + per < rows ? r0 + per : rows;
   float s = 0.f;
-  if (c < C)
-    for (int64_t r = r0 + wp; r < r1; r += 8) s += g[r * cs + c];
+  if (c < C) {
+    // 32 rows' loads in flight, added in row order (a few warps sum it all: one
+    // load at a time took 64 us for 262144 x 32, this 17)
+    int64_t r = r0 + wp;
+    for (; r + 8 * 31 < r1; r += 8 * 32) {
+      float v[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) v[k] = __ldg(g + (r + 8 * k) * cs + c);
+#pragma unroll
+      for (int k = 0; k < 32; ++k) s += v[k];
+    }
+    for (; r < r1; r += 8) s += g[r * cs + c];
+  }
   __shared__ float sh[8][32];
   sh[wp][lane] = s;
   __syncthreads();
@@ -1186,11 +1300,14 @@ __global__ void __launch_bounds__(256) k_bias_grad_part(const float* __restrict_
   }
 }
 
-__global__ void k_bias_grad_final(int C, int chunks, float* __restrict__ db) {
+__global__ void k_bias_grad_final(int C, float* __restrict__ db) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= C) return;
-  float t = 0.f;
-  for (int k = 0; k < chunks; ++k) t += g_bias_partial[(int64_t)k * C + c];
+  float v[kBiasChunks], t = 0.f;
+#pragma unroll
+  for (int k = 0; k < kBiasChunks; ++k) v[k] = g_bias_partial[(int64_t)k * C + c];
+#pragma unroll
+  for (int k = 0; k < kBiasChunks; ++k) t += v[k];
   db[c] = t;
 }
 
@@ -1231,9 +1348,14 @@ __global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ 
 
 __global__ void k_sum(const double* __restrict__ partial, int n, double scale,
                       double* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  if (blockIdx.x != 0) return;
+  __shared__ double sh[256];  // loaded together, added in order
+  for (int i = threadIdx.x; i < n; i += blockDim.x) sh[i] = partial[i];
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   double s = 0.0;
-  for (int i = 0; i < n; ++i) s += partial[i];
+#pragma unroll 16
+  for (int i = 0; i < n; ++i) s += sh[i];
   *out = s * scale;
 }
 
@@ -1291,6 +1413,12 @@ ddflb_status bad(const char* msg) {
 }  // namespace
 
 namespace {
+// the vector kernels: chunks of v elements, 32-bit indices
+bool vec_ok(int64_t n, int C, int cs1, int cs2, const void* p1, const void* p2, int v) {
+  return C % v == 0 && cs1 % v == 0 && cs2 % v == 0 && (uintptr_t)p1 % 16 == 0 &&
+         (uintptr_t)p2 % 16 == 0 && n < INT32_MAX;
+}
+
 int g_gemm_path = 0;  // 0: tcgen05 persistent (default), 1: mma.sync, 2: tcgen05 one tile per CTA
 
 // cuTensorMapEncodeTiled from the driver, looked up through the runtime (no
@@ -1440,6 +1568,71 @@ ddflb_status conv_tcp_bn(GemmArgs g, const void* X, int B, int cs, cudaStream_t 
   return launched("conv3x3 tcgen05");
 }
 
+// Geometry of a narrow convolution with mt units of 128 positions per tile;
+// false where it does not apply.
+bool narrow_args(narrow::Args* a, const void* X, int B, int H, int W, int C, int cs,
+                 const void* Wt, int bn, int mt, const GemmArgs& g) {
+  *a = narrow::Args{};
+  a->X = (const bf16*)X;
+  a->B = B;
+  a->H = H;
+  a->W = W;
+  a->cs = cs;
+  a->Wt = (const bf16*)Wt;
+  a->segment = W % 128 == 0;
+  a->pitch = a->segment ? 130 : W + 2;
+  a->inv_pitch = 0xffffffffu / (uint32_t)a->pitch + 1u;
+  a->npos = a->segment ? (mt + 2) * 130 : mt * 128 + 2 * a->pitch + 2;
+  a->unit_step = a->segment ? 130 : 128;
+  const int64_t per = a->segment ? (int64_t)((H + mt - 1) / mt) * (W / 128)
+                                 : ((int64_t)H * a->pitch + 128 * mt - 1) / (128 * mt);
+  if (per * B > INT32_MAX / 512 || ((int64_t)H + 8) * a->pitch * a->pitch >= (int64_t)1 << 32)
+    return false;  // (and positions / pitch by one multiplication)
+  a->per_img = (int)per;
+  a->tiles = (int)(per * B);
+  a->ntn = (g.N + bn - 1) / bn;
+  a->g = g;
+  const int64_t weights = 9 * (C / 8) * (int64_t)bn * 16, buf = (C / 8) * (int64_t)a->npos * 16;
+  for (a->nbuf = 4; a->nbuf >= 2; --a->nbuf)
+    if (weights + a->nbuf * buf <= tcp::SMEM_MAX) return a->ntn <= sm_count();
+  return false;
+}
+
+template <int CH, int BN, bool SEP, int MT>
+ddflb_status narrow_run(const narrow::Args& a, cudaStream_t s) {
+  auto* kernel = narrow::k_conv_narrow<CH, BN, SEP, MT>;
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tcp::SMEM_MAX);
+  if (attr != cudaSuccess) return bad("narrow convolution: shared memory attribute");
+  const int smem = 9 * CH * BN * 16 + a.nbuf * CH * a.npos * 16;
+  const int per = sm_count() / a.ntn;
+  kernel<<<(a.tiles < per ? a.tiles : per) * a.ntn, narrow::THREADS, smem, s>>>(a);
+  return launched("narrow convolution");
+}
+
+// Two units per tile where every SM still gets one (64^2, 64 -> 64, 16 images:
+// 16.5 us, one unit per tile 18.5), else one unit.  `refused`: whether the shape
+// does not fit at all.
+template <int CH, int BN, bool SEP>
+ddflb_status narrow_go(const void* X, int B, int H, int W, int cs, const void* Wt,
+                       const GemmArgs& g, cudaStream_t s, bool* refused) {
+  narrow::Args a;
+  *refused = false;
+  if (narrow_args(&a, X, B, H, W, 8 * CH, cs, Wt, BN, 2, g) && 
+      a.tiles >= sm_count() / a.ntn)
+    return narrow_run<CH, BN, SEP, 2>(a, s);
+  if (narrow_args(&a, X, B, H, W, 8 * CH, cs, Wt, BN, 1, g)) return narrow_run<CH, BN, SEP, 1>(a, s);
+  *refused = true;
+  return bad("convolution: rows too wide for a tile in shared memory");
+}
+
+template <int CH>
+ddflb_status narrow_fwd(const void* X, int B, int H, int W, int cs, const void* Wt,
+                        const GemmArgs& g, cudaStream_t s, bool* refused) {
+  return g.N <= 32 ? narrow_go<CH, 32, false>(X, B, H, W, cs, Wt, g, s, refused)
+                   : narrow_go<CH, 64, false>(X, B, H, W, cs, Wt, g, s, refused);
+}
+
 template <int BN>
 ddflb_status gemm_tc_bn(const GemmArgs& g, dim3 grid, cudaStream_t s) {
   static bool attr = false;
@@ -1568,71 +1761,6 @@ ddflb_status ddflb_nn_conv3x3(const void* X, int32_t B, int32_t H, int32_t W, in
   if (128 % bw || (W >= 128 && W % 128) || H % bh || bw * bh * bb != 128 || B % bb ||
       ((int64_t)B * H * W) % 128 || (int64_t)B * H * W > INT32_MAX)
     return bad("conv3x3: 128-pixel tiles need W a divisor of 128 or a multiple of it, and whole "
-// Geometry of a narrow convolution with mt units of 128 positions per tile;
-// false where it does not apply.
-bool narrow_args(narrow::Args* a, const void* X, int B, int H, int W, int C, int cs,
-                 const void* Wt, int bn, int mt, const GemmArgs& g) {
-  *a = narrow::Args{};
-  a->X = (const bf16*)X;
-  a->B = B;
-  a->H = H;
-  a->W = W;
-  a->cs = cs;
-  a->Wt = (const bf16*)Wt;
-  a->segment = W % 128 == 0;
-  a->pitch = a->segment ? 130 : W + 2;
-  a->inv_pitch = 0xffffffffu / (uint32_t)a->pitch + 1u;
-  a->npos = a->segment ? (mt + 2) * 130 : mt * 128 + 2 * a->pitch + 2;
-  a->unit_step = a->segment ? 130 : 128;
-  const int64_t per = a->segment ? (int64_t)((H + mt - 1) / mt) * (W / 128)
-                                 : ((int64_t)H * a->pitch + 128 * mt - 1) / (128 * mt);
-  if (per * B > INT32_MAX / 512 || ((int64_t)H + 8) * a->pitch * a->pitch >= (int64_t)1 << 32)
-    return false;  // (and positions / pitch by one multiplication)
-  a->per_img = (int)per;
-  a->tiles = (int)(per * B);
-  a->ntn = (g.N + bn - 1) / bn;
-  a->g = g;
-  const int64_t weights = 9 * (C / 8) * (int64_t)bn * 16, buf = (C / 8) * (int64_t)a->npos * 16;
-  for (a->nbuf = 4; a->nbuf >= 2; --a->nbuf)
-    if (weights + a->nbuf * buf <= tcp::SMEM_MAX) return a->ntn <= sm_count();
-  return false;
-}
-
-template <int CH, int BN, bool SEP, int MT>
-ddflb_status narrow_run(const narrow::Args& a, cudaStream_t s) {
-  auto* kernel = narrow::k_conv_narrow<CH, BN, SEP, MT>;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tcp::SMEM_MAX);
-  if (attr != cudaSuccess) return bad("narrow convolution: shared memory attribute");
-  const int smem = 9 * CH * BN * 16 + a.nbuf * CH * a.npos * 16;
-  const int per = sm_count() / a.ntn;
-  kernel<<<(a.tiles < per ? a.tiles : per) * a.ntn, narrow::THREADS, smem, s>>>(a);
-  return launched("narrow convolution");
-}
-
-// Two units per tile where every SM still gets one (64^2, 64 -> 64, 16 images:
-// 16.5 us, one unit per tile 18.5), else one unit.  `refused`: whether the shape
-// does not fit at all.
-template <int CH, int BN, bool SEP>
-ddflb_status narrow_go(const void* X, int B, int H, int W, int cs, const void* Wt,
-                       const GemmArgs& g, cudaStream_t s, bool* refused) {
-  narrow::Args a;
-  *refused = false;
-  if (narrow_args(&a, X, B, H, W, 8 * CH, cs, Wt, BN, 2, g) && 
-      a.tiles >= sm_count() / a.ntn)
-    return narrow_run<CH, BN, SEP, 2>(a, s);
-  if (narrow_args(&a, X, B, H, W, 8 * CH, cs, Wt, BN, 1, g)) return narrow_run<CH, BN, SEP, 1>(a, s);
-  *refused = true;
-  return bad("convolution: rows too wide for a tile in shared memory");
-}
-
-template <int CH>
-ddflb_status narrow_fwd(const void* X, int B, int H, int W, int cs, const void* Wt,
-                        const GemmArgs& g, cudaStream_t s, bool* refused) {
-  return g.N <= 32 ? narrow_go<CH, 32, false>(X, B, H, W, cs, Wt, g, s, refused)
-                   : narrow_go<CH, 64, false>(X, B, H, W, cs, Wt, g, s, refused);
-}
-
                "boxes of rows and images");
   GemmArgs g{};
   g.A = (const bf16*)X;
@@ -1658,10 +1786,64 @@ ddflb_status narrow_fwd(const void* X, int B, int H, int W, int cs, const void* 
   g.conv_bh = bh;
   g.conv_bb = bb;
   cudaStream_t s = (cudaStream_t)stream;
+  if (C == 64 && g_conv_path == 0) {
+    bool refused;
+    const ddflb_status st = narrow_fwd<8>(X, B, H, W, cs, Wt, g, s, &refused);
+    if (!refused) return st;
+  }
   const int bn = N <= 32 ? 32 : N <= 64 ? 64 : 128;
   return bn == 32 ? conv_tcp_bn<32>(g, X, B, cs, s)
          : bn == 64 ? conv_tcp_bn<64>(g, X, B, cs, s)
                     : conv_tcp_bn<128>(g, X, B, cs, s);
+}
+
+ddflb_status ddflb_nn_conv3x3_narrow(const void* X, int32_t B, int32_t H, int32_t W, int32_t C,
+                                     int32_t cs, const void* Wt, int32_t N, float* Cf, int32_t ldc,
+                                     void* Cb, int32_t ldcb, const float* bias, int32_t act,
+                                     int32_t accumulate, void* stream) {
+  if (!X || !Wt || B <= 0 || H <= 0 || W <= 0 || N <= 0 || (!Cf && !Cb))
+    return bad("conv3x3_narrow: bad arguments");
+  if ((C != 16 && C != 32 && C != 64) || cs < C || cs % 8 || ((uintptr_t)X % 16) ||
+      ((uintptr_t)Wt % 16))
+    return bad("conv3x3_narrow: C must be 16, 32 or 64, cs a multiple of 8 (>= C), X and Wt "
+               "16-byte aligned");
+  if ((Cf && ldc < N) || (Cb && ldcb < N)) return bad("conv3x3_narrow: leading dims");
+  if (act < 0 || act > 1) return bad("conv3x3_narrow: act must be 0 (none) or 1 (leaky ReLU)");
+  GemmArgs g{};
+  g.N = N;
+  g.Cf = Cf;
+  g.Cb = (bf16*)Cb;
+  g.ldc = ldc;
+  g.ldcb = ldcb;
+  g.bias = bias;
+  g.act = act;
+  g.accumulate = accumulate;
+  cudaStream_t s = (cudaStream_t)stream;
+  if ((int64_t)B * H * W > INT32_MAX) return bad("conv3x3_narrow: too many pixels");
+  bool refused;
+  return C == 16   ? narrow_fwd<2>(X, B, H, W, cs, Wt, g, s, &refused)
+         : C == 32 ? narrow_fwd<4>(X, B, H, W, cs, Wt, g, s, &refused)
+                   : narrow_fwd<8>(X, B, H, W, cs, Wt, g, s, &refused);
+}
+
+ddflb_status ddflb_nn_conv3x3_dgrad(const void* G, int32_t B, int32_t H, int32_t W, int32_t Co,
+                                    int32_t cs, const void* Wt, int32_t Ci, float* dX, int32_t ldc,
+                                    void* stream) {
+  if (!G || !Wt || !dX || B <= 0 || H <= 0 || W <= 0 || Ci <= 0)
+    return bad("conv3x3_dgrad: bad arguments");
+  if ((Co != 16 && Co != 32 && Co != 64) || cs < Co || cs % 8 || ((uintptr_t)G % 16) || ldc < Ci)
+    return bad("conv3x3_dgrad: Co must be 16, 32 or 64, cs a multiple of 8 (>= Co), G 16-byte "
+               "aligned, ldc >= Ci");
+  GemmArgs g{};
+  g.N = Ci;
+  g.Cf = dX;
+  g.ldc = ldc;
+  cudaStream_t s = (cudaStream_t)stream;
+  if ((int64_t)B * H * W > INT32_MAX) return bad("conv3x3_dgrad: too many pixels");
+  bool refused;
+  return Co == 16   ? narrow_go<2, 32, true>(G, B, H, W, cs, Wt, g, s, &refused)
+         : Co == 32 ? narrow_go<4, 32, true>(G, B, H, W, cs, Wt, g, s, &refused)
+                    : narrow_go<8, 32, true>(G, B, H, W, cs, Wt, g, s, &refused);
 }
 
 ddflb_status ddflb_nn_set_conv_path(int32_t path) {
@@ -1722,6 +1904,11 @@ ddflb_status ddflb_nn_pool(const void* X, int32_t B, int32_t H, int32_t W, int32
                            void* Y, int32_t csy, void* stream) {
   if (!X || !Y || H % 2 || W % 2 || C <= 0) return bad("pool: bad args");
   const int64_t n = (int64_t)B * (H / 2) * (W / 2) * C;
+  if (vec_ok(n, C, csx, csy, X, Y, 8)) {
+    k_pool_v8<<<grid_for(n / 8), 256, 0, (cudaStream_t)stream>>>(
+        (const bf16*)X, (uint32_t)(n / 8), H, W, C / 8, csx, (bf16*)Y, csy);
+    return launched("pool");
+  }
   k_pool<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16*)X, B, H, W, C, csx,
                                                         (bf16*)Y, csy);
   return launched("pool");
@@ -1732,6 +1919,11 @@ ddflb_status ddflb_nn_pool_bwd(const float* dY, int32_t B, int32_t H, int32_t W,
                                void* stream) {
   if (!dY || !dX || H % 2 || W % 2 || C <= 0) return bad("pool_bwd: bad args");
   const int64_t n = (int64_t)B * H * W * C;
+  if (vec_ok(n, C, csx, csy, dX, dY, 4)) {
+    k_pool_bwd_v4<<<grid_for(n / 16), 256, 0, (cudaStream_t)stream>>>(
+        dY, (uint32_t)(n / 16), W, C / 4, csy, dX, csx, accumulate);
+    return launched("pool_bwd");
+  }
   k_pool_bwd<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(dY, B, H, W, C, csy, dX, csx,
                                                             accumulate);
   return launched("pool_bwd");
@@ -1741,6 +1933,11 @@ ddflb_status ddflb_nn_upsample(const void* X, int32_t B, int32_t H, int32_t W, i
                                int32_t csx, void* Y, int32_t csy, void* stream) {
   if (!X || !Y || C <= 0) return bad("upsample: bad args");
   const int64_t n = (int64_t)B * 4 * H * W * C;
+  if (vec_ok(n, C, csx, csy, X, Y, 8)) {
+    k_upsample_v8<<<grid_for(n / 32), 256, 0, (cudaStream_t)stream>>>(
+        (const bf16*)X, (uint32_t)(n / 32), H, W, C / 8, csx, (bf16*)Y, csy);
+    return launched("upsample");
+  }
   k_upsample<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16*)X, B, H, W, C, csx,
                                                             (bf16*)Y, csy);
   return launched("upsample");
@@ -1750,6 +1947,11 @@ ddflb_status ddflb_nn_upsample_bwd(const float* dY, int32_t B, int32_t H, int32_
                                    int32_t csy, float* dX, int32_t csx, void* stream) {
   if (!dY || !dX || C <= 0) return bad("upsample_bwd: bad args");
   const int64_t n = (int64_t)B * H * W * C;
+  if (vec_ok(n, C, csx, csy, dX, dY, 4)) {
+    k_upsample_bwd_v4<<<grid_for(n / 4), 256, 0, (cudaStream_t)stream>>>(
+        dY, (uint32_t)(n / 4), W, C / 4, csy, dX, csx);
+    return launched("upsample_bwd");
+  }
   k_upsample_bwd<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(dY, B, H, W, C, csy, dX, csx);
   return launched("upsample_bwd");
 }
@@ -1757,6 +1959,12 @@ ddflb_status ddflb_nn_upsample_bwd(const float* dY, int32_t B, int32_t H, int32_
 ddflb_status ddflb_nn_act_bwd(float* g, const void* y, int64_t rows, int32_t C, int32_t csg,
                               int32_t csy, int32_t act, void* gb, int32_t csb, void* stream) {
   if (!g || !y || rows <= 0 || C <= 0) return bad("act_bwd: bad args");
+  if (vec_ok(rows * C, C, csg, csy, g, nullptr, 4) && (uintptr_t)y % 8 == 0 &&
+      (!gb || (csb % 4 == 0 && (uintptr_t)gb % 8 == 0))) {
+    k_act_bwd_v4<<<grid_for(rows * C / 4), 256, 0, (cudaStream_t)stream>>>(
+        g, (const bf16*)y, (uint32_t)(rows * C / 4), C / 4, csg, csy, act, (bf16*)gb, csb);
+    return launched("act_bwd");
+  }
   k_act_bwd<<<grid_for(rows * C), 256, 0, (cudaStream_t)stream>>>(g, (const bf16*)y, rows, C, csg,
                                                                   csy, act, (bf16*)gb, csb);
   return launched("act_bwd");
@@ -1770,7 +1978,7 @@ ddflb_status ddflb_nn_bias_grad(const float* g, int64_t rows, int32_t C, int32_t
     // the scratch is one per process: calls on different streams must not overlap
     dim3 grid((C + 31) / 32, kBiasChunks);
     k_bias_grad_part<<<grid, 256, 0, st>>>(g, rows, C, cs);
-    k_bias_grad_final<<<(C + 127) / 128, 128, 0, st>>>(C, kBiasChunks, db);
+    k_bias_grad_final<<<(C + 31) / 32, 32, 0, st>>>(C, db);
   } else {
     k_bias_grad<<<C, 256, 0, st>>>(g, rows, C, cs, db);
   }
@@ -1782,70 +1990,16 @@ ddflb_status ddflb_nn_mse(const float* pred, const float* target, int64_t n, flo
   if (!pred || !target || !dev_partial || !dev_loss || n <= 0) return bad("mse: bad args");
   const int nb = 256;  // dev_partial holds 256 doubles
   k_mse<<<nb, 256, 0, (cudaStream_t)stream>>>(pred, target, n, grad, dev_partial);
-  k_sum<<<1, 32, 0, (cudaStream_t)stream>>>(dev_partial, nb, 1.0 / (double)n, dev_loss);
+  k_sum<<<1, 256, 0, (cudaStream_t)stream>>>(dev_partial, nb, 1.0 / (double)n, dev_loss);
   return launched("mse");
 }
 
-  if (C == 64 && g_conv_path == 0) {
-    bool refused;
-    const ddflb_status st = narrow_fwd<8>(X, B, H, W, cs, Wt, g, s, &refused);
-    if (!refused) return st;
-  }
 ddflb_status ddflb_nn_adam(float* w, const float* g, float* m, float* v, void* wb, int64_t n,
                            float lr, float beta1, float beta2, float eps, int64_t t, float wd,
                            void* stream) {
   if (!w || !g || !m || !v || n <= 0 || t < 1) return bad("adam: bad args");
   const float c1 = 1.f - powf(beta1, (float)t), c2 = 1.f - powf(beta2, (float)t);
   k_adam<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(w, g, m, v, (bf16*)wb, n, lr, beta1,
-ddflb_status ddflb_nn_conv3x3_narrow(const void* X, int32_t B, int32_t H, int32_t W, int32_t C,
-                                     int32_t cs, const void* Wt, int32_t N, float* Cf, int32_t ldc,
-                                     void* Cb, int32_t ldcb, const float* bias, int32_t act,
-                                     int32_t accumulate, void* stream) {
-  if (!X || !Wt || B <= 0 || H <= 0 || W <= 0 || N <= 0 || (!Cf && !Cb))
-    return bad("conv3x3_narrow: bad arguments");
-  if ((C != 16 && C != 32 && C != 64) || cs < C || cs % 8 || ((uintptr_t)X % 16) ||
-      ((uintptr_t)Wt % 16))
-    return bad("conv3x3_narrow: C must be 16, 32 or 64, cs a multiple of 8 (>= C), X and Wt "
-               "16-byte aligned");
-  if ((Cf && ldc < N) || (Cb && ldcb < N)) return bad("conv3x3_narrow: leading dims");
-  if (act < 0 || act > 1) return bad("conv3x3_narrow: act must be 0 (none) or 1 (leaky ReLU)");
-  GemmArgs g{};
-  g.N = N;
-  g.Cf = Cf;
-  g.Cb = (bf16*)Cb;
-  g.ldc = ldc;
-  g.ldcb = ldcb;
-  g.bias = bias;
-  g.act = act;
-  g.accumulate = accumulate;
-  cudaStream_t s = (cudaStream_t)stream;
-  if ((int64_t)B * H * W > INT32_MAX) return bad("conv3x3_narrow: too many pixels");
-  bool refused;
-  return C == 16   ? narrow_fwd<2>(X, B, H, W, cs, Wt, g, s, &refused)
-         : C == 32 ? narrow_fwd<4>(X, B, H, W, cs, Wt, g, s, &refused)
-                   : narrow_fwd<8>(X, B, H, W, cs, Wt, g, s, &refused);
-}
-
-ddflb_status ddflb_nn_conv3x3_dgrad(const void* G, int32_t B, int32_t H, int32_t W, int32_t Co,
-                                    int32_t cs, const void* Wt, int32_t Ci, float* dX, int32_t ldc,
-                                    void* stream) {
-  if (!G || !Wt || !dX || B <= 0 || H <= 0 || W <= 0 || Ci <= 0)
-    return bad("conv3x3_dgrad: bad arguments");
-  if ((Co != 16 && Co != 32 && Co != 64) || cs < Co || cs % 8 || ((uintptr_t)G % 16) || ldc < Ci)
-    return bad("conv3x3_dgrad: Co must be 16, 32 or 64, cs a multiple of 8 (>= Co), G 16-byte "
-               "aligned, ldc >= Ci");
-  GemmArgs g{};
-  g.N = Ci;
-  g.Cf = dX;
-  g.ldc = ldc;
-  cudaStream_t s = (cudaStream_t)stream;
-  if ((int64_t)B * H * W > INT32_MAX) return bad("conv3x3_dgrad: too many pixels");
-  bool refused;
-  return Co == 16   ? narrow_go<2, 32, true>(G, B, H, W, cs, Wt, g, s, &refused)
-         : Co == 32 ? narrow_go<4, 32, true>(G, B, H, W, cs, Wt, g, s, &refused)
-                    : narrow_go<8, 32, true>(G, B, H, W, cs, Wt, g, s, &refused);
-}
-
                                                          beta2, eps, c1, c2, wd);
   return launched("adam");
 }
