@@ -537,6 +537,16 @@ ddflb_status ddflb_nn_conv3x3_narrow(const void* X, int32_t B, int32_t H, int32_
 ddflb_status ddflb_nn_conv3x3_dgrad(const void* G, int32_t B, int32_t H, int32_t W, int32_t Co,
                                     int32_t cs, const void* Wt, int32_t Ci, float* dX, int32_t ldc,
                                     void* stream);
+/* Weight gradient dW [Co][9 Ci] FP32 (tap-major) of Y = conv3x3(X, Wt) from X
+ * BF16 NHWC (Ci = 16 or a multiple of 32, channel stride csx) and dY = G BF16
+ * NHWC (Co a multiple of 8 up to 128, channel stride csg): FP32 sums over the
+ * pixels in at most `splits` slices, the slices added in a fixed order; partial:
+ * scratch of splits * Co * 9 Ci floats.  Where W is a multiple of 64,
+ * bit-identical to ddflb_nn_gemm with the same splits on the transposed
+ * gradient and the transposed im2col matrix. */
+ddflb_status ddflb_nn_conv3x3_wgrad(const void* X, int32_t B, int32_t H, int32_t W, int32_t Ci,
+                                    int32_t csx, const void* G, int32_t Co, int32_t csg, float* dW,
+                                    int32_t splits, float* partial, void* stream);
 /* Weights of the adjoint convolution: Wf[ci][t][co] = Wt[co][8 - t][ci]
  * (BF16, Wt [Co][9][Ci] -> Wf [Ci][9][Co]), so that dX = conv3x3(dY, Wf)
  * with C = Co and N = Ci is the input gradient of Y = conv3x3(X, Wt). */

@@ -907,6 +907,7 @@ __global__ void __launch_bounds__(tcp::THREADS, 1) k_gemm_tcp(
 }
 
 #include "ddflb_nn_narrow.cuh"
+#include "ddflb_nn_wgrad.cuh"
 
 // split-K: C = sum over slices z (fixed order) of partial[z]; then bias, act
 __global__ void k_splitk_reduce(const float* __restrict__ partial, int splits, int M, int N,
@@ -916,7 +917,15 @@ __global__ void k_splitk_reduce(const float* __restrict__ partial, int splits, i
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
     float v = 0.f;
-    for (int z = 0; z < splits; ++z) v += partial[(int64_t)z * total + i];
+    int z = 0;
+    for (; z + 8 <= splits; z += 8) {  // eight loads in flight, added in order
+      float q[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) q[k] = __ldg(partial + (int64_t)(z + k) * total + i);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v += q[k];
+    }
+    for (; z < splits; ++z) v += partial[(int64_t)z * total + i];
     const int r = (int)(i / N), c = (int)(i % N);
     if (bias) v += bias[c];
     v = act_fwd(v, act);
@@ -1844,6 +1853,66 @@ ddflb_status ddflb_nn_conv3x3_dgrad(const void* G, int32_t B, int32_t H, int32_t
   return Co == 16   ? narrow_go<2, 32, true>(G, B, H, W, cs, Wt, g, s, &refused)
          : Co == 32 ? narrow_go<4, 32, true>(G, B, H, W, cs, Wt, g, s, &refused)
                     : narrow_go<8, 32, true>(G, B, H, W, cs, Wt, g, s, &refused);
+}
+
+ddflb_status ddflb_nn_conv3x3_wgrad(const void* X, int32_t B, int32_t H, int32_t W, int32_t Ci,
+                                    int32_t csx, const void* G, int32_t Co, int32_t csg, float* dW,
+                                    int32_t splits, float* partial, void* stream) {
+  if (!X || !G || !dW || !partial || B <= 0 || H <= 0 || W <= 0 || splits < 1)
+    return bad("conv3x3_wgrad: bad arguments");
+  if ((Ci != 16 && Ci % 32) || Ci <= 0 || Co % 8 || Co <= 0 || Co > 128 || csx < Ci || csg < Co ||
+      csx % 8 || csg % 8 || ((uintptr_t)X % 16) || ((uintptr_t)G % 16) || ((uintptr_t)partial % 16))
+    return bad("conv3x3_wgrad: Ci must be 16 or a multiple of 32, Co a multiple of 8 up to 128, "
+               "the strides multiples of 8, X, G and partial 16-byte aligned");
+  wgrad::Args a{};
+  a.X = (const bf16*)X;
+  a.G = (const bf16*)G;
+  a.H = H;
+  a.W = W;
+  a.csx = csx;
+  a.csg = csg;
+  a.Ci = Ci;
+  a.Co = Co;
+  constexpr int U = wgrad::UNIT;
+  a.segment = W % U == 0;
+  a.pitch = W + 2;
+  a.inv_pitch = 0xffffffffu / (uint32_t)a.pitch + 1u;
+  const int64_t P = (int64_t)B * H * W;
+  const int64_t per = a.segment ? (int64_t)H * (W / U) : ((int64_t)H * a.pitch + U - 1) / U;
+  if (P > INT32_MAX || per * B > INT32_MAX / 512 ||
+      (!a.segment && ((int64_t)H + 8) * a.pitch * a.pitch >= (int64_t)1 << 32))
+    return bad("conv3x3_wgrad: image too large");
+  a.per_img = (int)per;
+  a.units = (int)(per * B);
+  // the GEMM's slices: ceil(P / splits) pixels, rounded up to 64
+  const int64_t kchunk = ((P + splits - 1) / splits + 63) / 64 * 64;
+  const int slices = (int)((P + kchunk - 1) / kchunk);
+  a.per_slice = a.segment ? (int)(kchunk / U) : (a.units + slices - 1) / slices;
+  a.ntn = Ci == 16 ? 1 : Ci / 32;
+  a.partial = partial;
+  const int chx = Ci == 16 ? 2 : 4;
+  const int buf = Co / 8 * U * 16 + chx * (U + 2) * 16;
+  // the MMAs read 128 rows of the gradient (16 planes) from a buffer's start
+  const int slack = buf < 16 * U * 16 ? 16 * U * 16 - buf : 0;
+  while ((1 << a.lane_bits) < Co / 8) ++a.lane_bits;
+  a.lanes = 1 << a.lane_bits;
+  a.nbuf = wgrad::MAXBUF;
+  while (a.nbuf > 2 && a.nbuf * buf + slack > tcp::SMEM_MAX / 2) --a.nbuf;  // two CTAs per SM
+  cudaStream_t s = (cudaStream_t)stream;
+  auto* kernel = chx == 2 ? wgrad::k_conv_wgrad<2> : wgrad::k_conv_wgrad<4>;
+  static const cudaError_t attr[2] = {
+      cudaFuncSetAttribute(wgrad::k_conv_wgrad<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           tcp::SMEM_MAX / 2),
+      cudaFuncSetAttribute(wgrad::k_conv_wgrad<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           tcp::SMEM_MAX / 2)};
+  if (attr[0] != cudaSuccess || attr[1] != cudaSuccess)
+    return bad("conv3x3_wgrad: shared memory attribute");
+  kernel<<<slices * a.ntn * 3, wgrad::THREADS, a.nbuf * buf + slack, s>>>(a);
+  ddflb_status st = launched("conv3x3_wgrad");
+  if (st != DDFLB_OK) return st;
+  k_splitk_reduce<<<grid_for((int64_t)Co * 9 * Ci), 256, 0, s>>>(partial, slices, Co, 9 * Ci, dW,
+                                                                 9 * Ci, nullptr, 0, 0);
+  return launched("conv3x3_wgrad sum");
 }
 
 ddflb_status ddflb_nn_set_conv_path(int32_t path) {

@@ -209,12 +209,19 @@ class UNet:
         _ck(self.lib.ddflb_nn_act_bwd(gout.ptr, vout.ptr, P, co, gout.cs, vout.cs, LEAKY, gbf, co,
                                       self.s))
         _ck(self.lib.ddflb_nn_bias_grad(gout.ptr, P, co, gout.cs, p["gb"].data_ptr(), self.s))
-        # dW [co][9ci] = g^T . im2col(x)
-        _ck(self.lib.ddflb_nn_transpose(gbf, P, co, co, gbT, self.s))
-        _ck(self.lib.ddflb_nn_im2col(vin.ptr, self.B, H, W, ci, vin.cs, self.colT.data_ptr(), 1,
-                                     self.s))
-        self._gemm(gbT, self.colT.data_ptr(), co, 9 * ci, P, P, P, Cf=p["gw"].data_ptr(),
-                   ldc=9 * ci, splits=self._splits(co, 9 * ci, P))
+        if self.implicit and (ci == 16 or ci % 32 == 0) and co % 8 == 0 and co <= 128:
+            # dW [co][9ci] from the activation and the gradient as they are
+            _ck(self.lib.ddflb_nn_conv3x3_wgrad(vin.ptr, self.B, H, W, ci, vin.cs, gbf, co, co,
+                                                p["gw"].data_ptr(),
+                                                self._splits(co, 9 * ci, P),
+                                                self.partial.data_ptr(), self.s))
+        else:
+            # dW = g^T . im2col(x)
+            _ck(self.lib.ddflb_nn_transpose(gbf, P, co, co, gbT, self.s))
+            _ck(self.lib.ddflb_nn_im2col(vin.ptr, self.B, H, W, ci, vin.cs, self.colT.data_ptr(),
+                                         1, self.s))
+            self._gemm(gbT, self.colT.data_ptr(), co, 9 * ci, P, P, P, Cf=p["gw"].data_ptr(),
+                       ldc=9 * ci, splits=self._splits(co, 9 * ci, P))
         if gin is None:
             return
         if self._implicit_ok(co, H, W):
