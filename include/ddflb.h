@@ -415,14 +415,12 @@ ddflb_status ddflb_batch_set_run(ddflb_batch* b, double tol, int32_t steps_per_l
  * 1e-10 capped at four times the cold steps.  Synchronises the stream. */
 ddflb_status ddflb_batch_set_instance_run(ddflb_batch* b, int32_t i, double tol,
                                           int64_t max_steps);
-/* How a chunk of steps is launched.  0 (default): one persistent cooperative
- * launch, every CTA walking its range of tiles step after step with a bounded
- * device-wide barrier between steps (suits many small lattices, where a
- * launch per step would cost more than the step).  1: one ordinary launch per
- * step with one CTA per tile, then a check kernel (one CTA per instance, idle
- * except at multiples of check_every) and at the end of the chunk a state-time
- * update, all captured in one graph per chunk; no barrier, more resident warps
- * (suits large batches).  Same results bit for bit.  The autotuner tries both. */
+/* How a chunk of steps is launched: 0 (default) = one persistent cooperative
+ * launch with a device-wide barrier between steps; 1 = ordinary launches
+ * captured in a graph, the stream as the barrier: two steps per launch between
+ * the residual checks (one warp per strip of an instance), single steps with one
+ * CTA per tile around them (suits large batches).  Same results bit for bit.
+ * The autotuner tries both. */
 ddflb_status ddflb_batch_set_schedule(ddflb_batch* b, int32_t schedule);
 ddflb_status ddflb_batch_get_schedule(const ddflb_batch* b, int32_t* schedule);
 /* Tile shape (32x4, 64x2, 128x1, 32x8, 64x4, 128x2, 256x1) and CTAs per SM

@@ -270,7 +270,7 @@ int choose_march_rows(const ddflb_ctx* c) {
   // while the last ones finish (FP32 8192^2, rows 16 / 32 / 64 / 128: 878, 853,
   // 870, 1023 us per step; 4096^2: 231, 237, 261, 325)
   const double slots = 152 * 15;
-  const int strips = (P.nx + kMarchStrip - 1) / kMarchStrip;
+  const int strips = march_strips(c->L.P_bc, P.nx);
   double best = 1e300;
   int rows = 16;
   for (int r : {8, 12, 16, 24, 32, 48, 64}) {

@@ -31,6 +31,7 @@
 #include "../../include/ddflb.h"
 #include "ddflb_device.cuh"
 #include "ddflb_internal.h"
+#include "ddflb_march.cuh"
 
 namespace ddflb {
 
@@ -58,7 +59,7 @@ struct BatchStatus {
   int64_t state_time;    // state time of the instance's current state when frozen
   long long init_time;   // state time at which the instance was (re)initialised
   int32_t flags;         // DDFLB_INST_CONVERGED | DDFLB_INST_DIVERGED | DDFLB_INST_CAPPED
-  int32_t pad;
+  int32_t buf;           // buffer that holds the state of a frozen instance
   double tol;            // this instance's tolerance (< 0: the batch's)
   int64_t max_steps;     // freeze after this many steps since init (0: no limit)
 };
@@ -79,6 +80,7 @@ struct BatchArgs {
   int ntiles;
   int tile_x, tile_y;
   int nsteps;
+  int src;  // buffer of the state at the start of the chunk
   int check_every;
   double tol;
   int scalar_residual;  // freeze only when the scalar residual is below tol too
@@ -215,8 +217,9 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 
 // Check of instance i after the step from state time t (a multiple of K): the
 // fixed-order reduction of its tiles' sums, then the freeze decision
-// (converged, diverged, or at its own step limit).  Called by one whole CTA.
-__device__ void check_instance(const BatchArgs& A, int i, int64_t t, double* sh) {
+// (converged, diverged, or at its own step limit).  dst: the buffer the step wrote.
+// Called by one whole CTA.
+__device__ void check_instance(const BatchArgs& A, int i, int64_t t, int dst, double* sh) {
   if (__ldcg(&A.ist[i].flags) != 0 || t - A.check_every < __ldcg(&A.ist[i].init_time)) return;
   const int b = A.inst[i].tile_begin, e = A.inst[i].tile_end;
   double v[kParts];
@@ -231,6 +234,7 @@ __device__ void check_instance(const BatchArgs& A, int i, int64_t t, double* sh)
     st.mass_dev = v[2];
     const double ru = v[0] > 0.0 ? sqrt(v[1] / v[0]) / A.check_every : 0.0;
     const double rp = v[3] > 0.0 ? sqrt(v[4] / v[3]) / A.check_every : 0.0;
+    st.buf = dst;
     st.residual_phi = rp;
     st.residual = A.scalar_residual ? fmax(ru, rp) : ru;
     const double tol = st.tol >= 0.0 ? st.tol : A.tol;
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(256, 4) k_batch(BatchArgs A) {
   int cur = -1;
   for (int s = 0; s < A.nsteps; ++s) {
     const int64_t t = t0 + s;
-    const int src = (int)(t & 1);
+    const int src = (A.src + s) & 1;
     // at every multiple of K: compare u with the snapshot from K steps earlier
     // (instances initialised at least K steps ago), then take the next snapshot
     const bool snap = A.check_every > 0 && t % A.check_every == 0;
@@ -327,7 +331,7 @@ __global__ void __launch_bounds__(256, 4) k_batch(BatchArgs A) {
     }
     if (check_t) {
       if (!grid_barrier(A.sync, A.timeout_ns)) return;
-      for (int i = blockIdx.x; i < A.ninst; i += gridDim.x) check_instance(A, i, t, sh);
+      for (int i = blockIdx.x; i < A.ninst; i += gridDim.x) check_instance(A, i, t, src ^ 1, sh);
       cur = -1;  // re-read the activity flags
     }
     if (s == 0 && (int)blockIdx.x == A.skip_block) return;  // test hook: never arrive
@@ -336,17 +340,16 @@ __global__ void __launch_bounds__(256, 4) k_batch(BatchArgs A) {
   if (blockIdx.x == 0 && threadIdx.x == 0) A.sync->step = t0 + A.nsteps;
 }
 
-// Schedule 1: one ordinary launch per time step, one CTA per tile, then (idle
-// except at check steps) the sums and check kernels and, at the end of a
-// chunk, the state-time update, all captured in one graph per chunk.  No
-// device-wide barrier: the stream orders the steps.  Step s of the chunk
-// advances the state from time sync->step + s.  The node update carries no
-// check code; at most 56 registers, so 9 CTAs of 128 threads stay resident.
+// Schedule 1: ordinary launches, ordered by the stream, captured in one graph
+// per chunk: two steps per launch (k_batch_march) between the check steps, and
+// around them single steps (k_batch_tile, one CTA per tile), each check step
+// followed by the sums and the check.  Step s of the chunk advances the state
+// from time sync->step + s.  The node update carries no check code; at most 56
+// registers, so 9 CTAs of 128 threads stay resident.
 template <typename S>
-__global__ void __maxnreg__(56) k_batch_tile(BatchArgs A, int s) {
+__global__ void __maxnreg__(56) k_batch_tile(BatchArgs A, int src) {
   __shared__ BatchInst sI;
   __shared__ int sActive;
-  const int64_t t = A.sync->step + s;
   const int4 T = __ldg(&A.tiles[blockIdx.x]);
   const int* srcw = (const int*)(A.inst + T.x);
   int* dstw = (int*)&sI;
@@ -355,7 +358,6 @@ __global__ void __maxnreg__(56) k_batch_tile(BatchArgs A, int s) {
   __syncthreads();
   if (!sActive) return;  // uniform over the CTA
   const LbParams& sP = sI.P;
-  const int src = (int)(t & 1);
   const int tx = threadIdx.x % A.tile_x, ty = threadIdx.x / A.tile_x;
   const int x = T.y + tx, y = T.z + ty;
   const bool in_x = sI.bc == BC_CHANNEL ? x < sP.nx : (x >= 1 && x < sP.nx - 1);
@@ -376,18 +378,15 @@ __global__ void __maxnreg__(56) k_batch_tile(BatchArgs A, int s) {
 // At a check step (state time t a multiple of K, after the step from t): the
 // residual sums of each tile from the state at time t, read back from the
 // step's source buffer (the step wrote the other one), and the new snapshot.
-// A grid of a few CTAs per SM walks the tiles; at other steps it returns.
+// A grid of a few CTAs per SM walks the tiles.
 template <typename S>
-__global__ void __launch_bounds__(256) k_batch_sums(BatchArgs A, int s) {
+__global__ void __launch_bounds__(256) k_batch_sums(BatchArgs A, int s, int src) {
   __shared__ BatchInst sI;
   __shared__ double sh[8];
   __shared__ int sActive;
   __shared__ long long sInit;
   const int64_t t = A.sync->step + s;
-  const bool snap = A.check_every > 0 && t % A.check_every == 0;
-  if (!snap) return;
   const LbParams& sP = sI.P;
-  const int src = (int)(t & 1);
   const int tx = threadIdx.x % A.tile_x, ty = threadIdx.x / A.tile_x;
   int cur = -1;
   for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x) {
@@ -429,13 +428,38 @@ __global__ void __launch_bounds__(256) k_batch_sums(BatchArgs A, int s) {
   }
 }
 
-// The checks after step s of a chunk (a no-op unless its state time is a
-// positive multiple of K): one CTA per instance.
-__global__ void __launch_bounds__(256) k_batch_check(BatchArgs A, int s) {
+// The checks after step s of a chunk (whose state time is a positive multiple of
+// K): one CTA per instance.
+__global__ void __launch_bounds__(256) k_batch_check(BatchArgs A, int s, int dst) {
   __shared__ double sh[8];
-  const int64_t t = A.sync->step + s;
-  if (!(A.check_every > 0 && t > 0 && t % A.check_every == 0)) return;
-  check_instance(A, blockIdx.x, t, sh);
+  check_instance(A, blockIdx.x, A.sync->step + s, dst, sh);
+}
+
+// Two steps of every active instance: one warp per item (instance, strip, rows),
+// as k_march2, with the instance's parameters and constants in shared memory.
+// 512 uneven cavities, FP32, 500 steps: 376 ms a pass with their initialisation
+// and fields; the persistent launch of single steps, at 0.79 of the copy
+// bandwidth, 526.
+template <typename S, int BC>
+__global__ void __launch_bounds__(32, kMarchWarps<S, BC>)
+    k_batch_march(BatchArgs A, const int4* __restrict__ items, const PairConst* __restrict__ consts,
+                  int src) {
+  extern __shared__ __align__(128) unsigned char march_shared[];
+  __shared__ __align__(8) uint64_t s_bar[PairIo<S>::STAGES];
+  __shared__ float s_wall[12];
+  __shared__ BatchInst sI;
+  __shared__ PairConst sK;
+  const int4 T = __ldg(&items[blockIdx.x]);
+  if (__ldcg(&A.ist[T.x].flags) != 0) return;
+  for (int w = threadIdx.x; w < (int)(sizeof(BatchInst) / 4); w += 32)
+    ((int*)&sI)[w] = __ldg((const int*)(A.inst + T.x) + w);
+  for (int w = threadIdx.x; w < (int)(sizeof(PairConst) / 4); w += 32)
+    ((int*)&sK)[w] = __ldg((const int*)(consts + T.x) + w);
+  __syncwarp();
+  const S* fin = (const S*)sI.buf[src];
+  S* fout = (S*)sI.buf[src ^ 1];
+  march_strip<S, BC>(sI.P, sK, fin, fin + sI.goff, fout, fout + sI.goff, T.y, T.z, T.w,
+                     march_shared, s_bar, s_wall, &A.sync->err);
 }
 
 __global__ void k_batch_advance(BatchSync* sync, int nsteps) {
@@ -474,8 +498,10 @@ constexpr int kNumShapes = 7;
 
 struct BLayout {
   std::vector<size_t> off_buf0, off_buf1, off_uprev;
-  size_t off_inst, off_tiles, off_part, off_status, off_sync, total;
+  size_t off_inst, off_tiles, off_part, off_status, off_sync, off_items, off_consts, total;
   int max_tiles;
+  int item_rows;        // rows per item of the two-step launches
+  int item_begin[4];    // items by boundary kind: [item_begin[bc], item_begin[bc + 1])
 };
 
 int count_tiles(int n, const ddflb_params* p, int tx, int ty) {
@@ -502,6 +528,23 @@ BLayout blayout(int n, const ddflb_params* p) {
   L.off_part = o; o += al((size_t)mt * kParts * sizeof(double));
   L.off_status = o; o += al(n * sizeof(BatchStatus));
   L.off_sync = o; o += al(sizeof(BatchSync));
+  // rows per item: as for one lattice, waves of 12 warps an SM and most of an
+  // item's time at the end (ddflb_api.cu)
+  auto items = [&](int r) {
+    int64_t k = 0;
+    for (int i = 0; i < n; ++i) k += (int64_t)march_strips(p[i].bc, p[i].nx) * ((p[i].ny + r - 1) / r);
+    return k;
+  };
+  double best = 1e300;
+  for (int r : {8, 12, 16, 24, 32, 48, 64}) {
+    const double cost = ((double)items(r) / (152 * 12) + 1.0) * (r + 3);
+    if (cost < best) {
+      best = cost;
+      L.item_rows = r;
+    }
+  }
+  L.off_items = o; o += al((size_t)items(L.item_rows) * sizeof(int4));
+  L.off_consts = o; o += al(n * sizeof(PairConst));
   L.total = o;
   return L;
 }
@@ -524,13 +567,20 @@ struct ddflb_batch {
   long long timeout_ns;
   int skip_block;
   int64_t step;  // host mirror of the global state time
+  int cur;       // buffer of the active instances' current state
   BatchInst* d_inst;
   int4* d_tiles;
   double* d_part;
   BatchStatus* d_status;
   BatchSync* d_sync;
-  cudaGraphExec_t graph;
-  int graph_chunk;
+  // captured chunks: by steps, buffer at the start and (schedule 1) the state
+  // time modulo check_every, which fixes the launches; a few at a time
+  struct Graph {
+    int steps, cur;
+    int64_t phase;
+    cudaGraphExec_t exec;
+  };
+  std::vector<Graph> graphs;
   bool graph_failed;
   std::vector<double> inst_tol;   // per-instance tolerance (< 0: the batch's)
   std::vector<int64_t> inst_cap;  // per-instance step limit (0: none)
@@ -540,6 +590,13 @@ struct ddflb_batch {
 };
 
 namespace {
+
+constexpr size_t kMaxGraphs = 8;
+
+void drop_graphs(ddflb_batch* b) {
+  for (auto& g : b->graphs) cudaGraphExecDestroy(g.exec);
+  b->graphs.clear();
+}
 
 ddflb_status upload_tiles(ddflb_batch* b) {
   std::vector<int4> tiles;
@@ -559,7 +616,28 @@ ddflb_status upload_tiles(ddflb_batch* b) {
     I.tile_end = (int)tiles.size();
   }
   b->ntiles = (int)tiles.size();
-  cudaError_t e = cudaMemcpyAsync(b->d_inst, inst.data(), inst.size() * sizeof(BatchInst),
+  // items of the two-step launches, by boundary kind, and the packed constants
+  std::vector<int4> items;
+  std::vector<PairConst> consts(b->n);
+  for (int bc = 0; bc < 3; ++bc) {
+    b->lay.item_begin[bc] = (int)items.size();
+    for (int i = 0; i < b->n; ++i) {
+      if (b->p[i].bc != bc) continue;
+      consts[i] = make_pair_const(b->lp[i]);
+      const int r = b->lay.item_rows;
+      for (int y = 0; y < b->p[i].ny; y += r)
+        for (int k = 0; k < march_strips(bc, b->p[i].nx); ++k)
+          items.push_back(make_int4(i, k, y, std::min(y + r, b->p[i].ny)));
+    }
+  }
+  b->lay.item_begin[3] = (int)items.size();
+  cudaError_t e = cudaMemcpyAsync(b->ws + b->lay.off_items, items.data(),
+                                  items.size() * sizeof(int4), cudaMemcpyHostToDevice, b->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->ws + b->lay.off_consts, consts.data(), b->n * sizeof(PairConst),
+                        cudaMemcpyHostToDevice, b->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->d_inst, inst.data(), inst.size() * sizeof(BatchInst),
                                   cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->d_tiles, tiles.data(), tiles.size() * sizeof(int4),
@@ -599,15 +677,13 @@ ddflb_status configure(ddflb_batch* b, int tx, int ty, int bps) {
   b->blocks_per_sm = bps > 0 ? std::min(bps, occ) : occ;
   b->grid = b->blocks_per_sm * nsm;
   b->sums_grid = 4 * nsm;
-  if (b->graph) {
-    cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-  }
+  drop_graphs(b);
   return upload_tiles(b);
 }
 
 BatchArgs args_for(ddflb_batch* b, int nsteps) {
   BatchArgs A;
+  A.src = b->cur;
   A.inst = b->d_inst;
   A.ninst = b->n;
   A.tiles = b->d_tiles;
@@ -626,25 +702,64 @@ BatchArgs args_for(ddflb_batch* b, int nsteps) {
   return A;
 }
 
-cudaError_t launch_chunk(ddflb_batch* b, cudaStream_t s, int nsteps) {
+template <typename S, int BC>
+cudaError_t launch_march(ddflb_batch* b, cudaStream_t s, const BatchArgs& A, int src) {
+  const int first = b->lay.item_begin[BC], count = b->lay.item_begin[BC + 1] - first;
+  if (count == 0) return cudaSuccess;
+  k_batch_march<S, BC><<<count, 32, march_smem<S>(BC), s>>>(
+      A, (const int4*)(b->ws + b->lay.off_items) + first,
+      (const PairConst*)(b->ws + b->lay.off_consts), src);
+  return cudaGetLastError();
+}
+
+template <typename S>
+cudaError_t launch_two(ddflb_batch* b, cudaStream_t s, const BatchArgs& A, int src) {
+  cudaError_t e = launch_march<S, BC_PERIODIC>(b, s, A, src);
+  if (e == cudaSuccess) e = launch_march<S, BC_CAVITY>(b, s, A, src);
+  return e == cudaSuccess ? launch_march<S, BC_CHANNEL>(b, s, A, src) : e;
+}
+
+// One chunk of nsteps steps from state time t0 and buffer b->cur; *end: the
+// buffer of the state after it.
+cudaError_t launch_chunk(ddflb_batch* b, cudaStream_t s, int nsteps, int64_t t0, int* end) {
   BatchArgs A = args_for(b, nsteps);
   if (b->schedule == 1) {
-    // one launch per step (+ the check kernel), then the state-time update
     const dim3 tb(b->tile_x * b->tile_y);
     void* sums = b->storage == 0 ? (void*)k_batch_sums<float>
                : b->storage == 1 ? (void*)k_batch_sums<__half> : (void*)k_batch_sums<__nv_bfloat16>;
-    for (int k = 0; k < nsteps; ++k) {
-      void* targs[] = {&A, &k};
-      cudaError_t e = cudaLaunchKernel(batch_kernel(b->storage, 1, b->bcs), dim3(b->ntiles), tb, targs, 0, s);
-      if (e == cudaSuccess) e = cudaLaunchKernel(sums, dim3(b->sums_grid), tb, targs, 0, s);
+    const int64_t K = b->p[0].check_every;
+    int cur = b->cur;
+    auto check_at = [&](int64_t t) { return K > 0 && t % K == 0; };
+    for (int k = 0; k < nsteps; cur ^= 1) {
+      const int64_t t = t0 + k;
+      cudaError_t e;
+      if (k + 1 < nsteps && !check_at(t) && !check_at(t + 1)) {
+        e = b->storage == 0   ? launch_two<float>(b, s, A, cur)
+            : b->storage == 1 ? launch_two<__half>(b, s, A, cur)
+                              : launch_two<__nv_bfloat16>(b, s, A, cur);
+        if (e != cudaSuccess) return e;
+        k += 2;
+        continue;
+      }
+      void* targs[] = {&A, &cur};
+      e = cudaLaunchKernel(batch_kernel(b->storage, 1, b->bcs), dim3(b->ntiles), tb, targs, 0, s);
       if (e != cudaSuccess) return e;
-      k_batch_check<<<b->n, 256, 0, s>>>(A, k);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
+      if (check_at(t)) {  // (t = 0: the first snapshot)
+        void* sargs[] = {&A, &k, &cur};
+        e = cudaLaunchKernel(sums, dim3(b->sums_grid), tb, sargs, 0, s);
+        if (e == cudaSuccess && t > 0) {
+          k_batch_check<<<b->n, 256, 0, s>>>(A, k, cur ^ 1);
+          e = cudaGetLastError();
+        }
+        if (e != cudaSuccess) return e;
+      }
+      ++k;
     }
+    *end = cur;
     k_batch_advance<<<1, 32, 0, s>>>(b->d_sync, nsteps);
     return cudaGetLastError();
   }
+  *end = (b->cur + nsteps) & 1;
   void* kargs[] = {&A};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(b->grid);
@@ -659,18 +774,37 @@ cudaError_t launch_chunk(ddflb_batch* b, cudaStream_t s, int nsteps) {
   return cudaLaunchKernelExC(&cfg, batch_kernel(b->storage, 0, b->bcs), kargs);
 }
 
-// Capture one chunk launch into a graph (on a private stream) for replay.
-void build_graph(ddflb_batch* b, int nsteps) {
-  if (b->graph_failed) return;
+// The buffer of the state after nsteps steps (as launch_chunk arranges them).
+int chunk_end(const ddflb_batch* b, int nsteps) {
+  const int64_t K = b->p[0].check_every;
+  if (b->schedule != 1) return (b->cur + nsteps) & 1;
+  int cur = b->cur;
+  auto check_at = [&](int64_t t) { return K > 0 && t % K == 0; };
+  for (int k = 0; k < nsteps; cur ^= 1) {
+    const int64_t t = b->step + k;
+    k += k + 1 < nsteps && !check_at(t) && !check_at(t + 1) ? 2 : 1;
+  }
+  return cur;
+}
+
+// The chunk launch as a graph (captured on a private stream), from the few kept
+// or newly built; null where capture is unavailable.
+cudaGraphExec_t chunk_graph(ddflb_batch* b, int nsteps) {
+  const int64_t K = b->p[0].check_every;
+  const int64_t phase = b->schedule == 1 && K > 0 ? (b->step == 0 ? -1 : b->step % K) : 0;
+  for (auto& g : b->graphs)
+    if (g.steps == nsteps && g.cur == b->cur && g.phase == phase) return g.exec;
+  if (b->graph_failed) return nullptr;
   cudaStream_t cs;
   if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
     b->graph_failed = true;
-    return;
+    return nullptr;
   }
   cudaGraph_t g = nullptr;
+  int end;
   bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
   if (ok) {
-    ok = launch_chunk(b, cs, nsteps) == cudaSuccess;
+    ok = launch_chunk(b, cs, nsteps, b->step, &end) == cudaSuccess;
     ok = (cudaStreamEndCapture(cs, &g) == cudaSuccess) && ok;
   }
   cudaGraphExec_t ex = nullptr;
@@ -680,10 +814,15 @@ void build_graph(ddflb_batch* b, int nsteps) {
   cudaGetLastError();  // clear a capture error, if any
   if (!ok) {
     b->graph_failed = true;
-    return;
+    return nullptr;
   }
-  b->graph = ex;
-  b->graph_chunk = nsteps;
+  if (b->graphs.size() == kMaxGraphs) {
+    cudaStreamSynchronize(b->stream);  // (it may still be running)
+    cudaGraphExecDestroy(b->graphs.front().exec);
+    b->graphs.erase(b->graphs.begin());
+  }
+  b->graphs.push_back({nsteps, b->cur, phase, ex});
+  return ex;
 }
 
 ddflb_status check_sync_error(ddflb_batch* b) {
@@ -751,7 +890,7 @@ ddflb_status ddflb_batch_create(int32_t n, const ddflb_params* p, void* ws, size
   b->d_part = (double*)(b->ws + b->lay.off_part);
   b->d_status = (BatchStatus*)(b->ws + b->lay.off_status);
   b->d_sync = (BatchSync*)(b->ws + b->lay.off_sync);
-  b->graph = nullptr;
+  b->cur = 0;
   b->graph_failed = false;
   b->schedule = 0;
   cudaError_t e = cudaMemsetAsync(b->d_sync, 0, sizeof(BatchSync), b->stream);
@@ -793,10 +932,7 @@ ddflb_status ddflb_batch_set_run(ddflb_batch* b, double tol, int32_t steps_per_l
   b->scalar_residual = scalar_residual != 0;
   b->chunk = steps_per_launch;
   b->timeout_ns = (long long)(barrier_timeout_s * 1e9);
-  if (b->graph) {
-    cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-  }
+  drop_graphs(b);
   return DDFLB_OK;
 }
 
@@ -867,7 +1003,7 @@ ddflb_status ddflb_batch_init(ddflb_batch* b, int32_t i, const float* rho, const
   L.stream = b->stream;
   InitPtrs in{rho, ux, uy, phi, grads};
   // the instance joins at the batch's current state time
-  const size_t off = (b->step & 1) ? b->lay.off_buf1[i] : b->lay.off_buf0[i];
+  const size_t off = b->cur ? b->lay.off_buf1[i] : b->lay.off_buf0[i];
   char* f = b->ws + off;
   char* g = f + 9 * (size_t)L.P.plane * esz(p.storage);
   cudaError_t e = launch_init(L, in, f, g);
@@ -895,15 +1031,14 @@ ddflb_status ddflb_batch_step(ddflb_batch* b, int64_t n) {
   int64_t left = n;
   while (left > 0) {
     const int k = (int)std::min<int64_t>(left, b->chunk);
-    if (k == b->chunk && !b->graph) build_graph(b, k);
-    cudaError_t e;
-    if (k == b->chunk && b->graph)
-      e = cudaGraphLaunch(b->graph, b->stream);
-    else
-      e = launch_chunk(b, b->stream, k);
+    cudaGraphExec_t ex = k == b->chunk ? chunk_graph(b, k) : nullptr;
+    int end = chunk_end(b, k);
+    const cudaError_t e =
+        ex ? cudaGraphLaunch(ex, b->stream) : launch_chunk(b, b->stream, k, b->step, &end);
     if (e != cudaSuccess) return bcuda(e, "batch step launch");
     left -= k;
     b->step += k;
+    b->cur = end;
   }
   return DDFLB_OK;
 }
@@ -915,7 +1050,7 @@ ddflb_status ddflb_batch_fields(ddflb_batch* b, int32_t i, float* rho, float* ux
   cudaError_t e = cudaMemcpyAsync(&s, b->d_status + i, sizeof s, cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bcuda(e, "batch fields status");
-  const int64_t t = s.flags ? s.state_time : b->step;
+  const int buf = s.flags ? s.buf : b->cur;
   Launch L;
   L.P = b->lp[i];
   L.P_bc = b->p[i].bc;
@@ -923,7 +1058,7 @@ ddflb_status ddflb_batch_fields(ddflb_batch* b, int32_t i, float* rho, float* ux
   L.force = false;
   L.block = dim3(128, 1, 1);
   L.stream = b->stream;
-  const char* f = b->ws + ((t & 1) ? b->lay.off_buf1[i] : b->lay.off_buf0[i]);
+  const char* f = b->ws + (buf ? b->lay.off_buf1[i] : b->lay.off_buf0[i]);
   const char* g = f + 9 * (size_t)L.P.plane * esz(b->p[i].storage);
   FieldPtrs fp{{rho, ux, uy, phi, sxx, sxy, syy, omega}};
   e = launch_fields(L, f, g, fp);
@@ -951,10 +1086,7 @@ ddflb_status ddflb_batch_stats(ddflb_batch* b, double* residual, int32_t* flags,
 ddflb_status ddflb_batch_debug_skip_barrier(ddflb_batch* b, int32_t block) {
   if (!b) return bfail(DDFLB_EINVAL, "NULL batch");
   b->skip_block = block;
-  if (b->graph) {
-    cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-  }
+  drop_graphs(b);
   return DDFLB_OK;
 }
 
@@ -999,9 +1131,10 @@ ddflb_status ddflb_batch_autotune(ddflb_batch* b, int32_t trial_steps, int32_t* 
         rs = configure(b, kShapes[k][0], kShapes[k][1], b->blocks_per_sm / 2);
         if (rs != DDFLB_OK) break;
       }
-      e = launch_chunk(b, s, trial_steps);
+      int end;  // (from state time 1: the launches between two checks)
+      e = launch_chunk(b, s, trial_steps, 1, &end);
       if (e == cudaSuccess) e = cudaEventRecord(e0, s);
-      if (e == cudaSuccess) e = launch_chunk(b, s, trial_steps);
+      if (e == cudaSuccess) e = launch_chunk(b, s, trial_steps, 1, &end);
       if (e == cudaSuccess) e = cudaEventRecord(e1, s);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms = 0.f;
@@ -1041,6 +1174,7 @@ ddflb_status ddflb_batch_autotune(ddflb_batch* b, int32_t trial_steps, int32_t* 
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return bcuda(e, "autotune reset");
   b->step = 0;
+  b->cur = 0;
   if (tile_x) *tile_x = bx;
   if (tile_y) *tile_y = by;
   if (blocks_per_sm) *blocks_per_sm = bb;
@@ -1049,7 +1183,7 @@ ddflb_status ddflb_batch_autotune(ddflb_batch* b, int32_t trial_steps, int32_t* 
 }
 
 ddflb_status ddflb_batch_destroy(ddflb_batch* b) {
-  if (b && b->graph) cudaGraphExecDestroy(b->graph);
+  if (b) drop_graphs(b);
   delete b;
   return DDFLB_OK;
 }

@@ -10,6 +10,10 @@
 namespace ddflb {
 
 constexpr int kMarchStrip = 60;  // columns of a strip of the two-step kernel
+inline int march_strips(int bc, int nx) {
+  if (bc == BC_CAVITY) return nx <= 64 ? 1 : 1 + (nx - 64 + kMarchStrip - 1) / kMarchStrip;
+  return (nx + kMarchStrip - 1) / kMarchStrip;
+}
 constexpr int64_t kMarchMinNodes = (int64_t)1 << 21;  // smallest lattice it is used for
 constexpr int kReduceThreads = 256;
 constexpr int kReduceBlocks = 608;  // 4 per SM on a 152-SM GB300; fixed for deterministic sums

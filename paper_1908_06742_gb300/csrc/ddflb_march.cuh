@@ -96,7 +96,9 @@ __device__ __forceinline__ F2 from_right(F2 v) {
   return make_float2(v.y, __shfl_down_sync(0xffffffffu, v.x, 1));
 }
 
-constexpr int kMarchHalo = 2;  // columns on each side of a strip computed for it only
+// warps per SM (the register budget: 128 at 16, 168 at 12)
+template <typename S, int BC>
+constexpr int kMarchWarps = sizeof(S) == 4 && BC != BC_PERIODIC ? 12 : 16;
 
 template <typename S>
 constexpr size_t march_smem(int bc) {
@@ -125,37 +127,42 @@ constexpr size_t march_smem(int bc) {
 // 79, 311 instructions per node and step against 553.  FP16 16384^2: 108 against
 // 91 of k_step_quad (16 warps an SM; 12: 97, 20 with spills: 78).  The walled
 // FP32 forms keep 12 warps (4096^2 cavity: 67; at 16, with spills: 60).
+//
+// `strip` and rows [y0, y1) name the strip and chunk; shared: march_smem() bytes;
+// bars: STAGES mbarriers; wall: 12 floats; *timeout is set if a copy fails to arrive.
 template <typename S, int BC>
-__global__ void __launch_bounds__(32, sizeof(S) == 4 && BC != BC_PERIODIC ? 12 : 16)
-    k_march2(LbParams P, PairConst K, const S* __restrict__ fin, const S* __restrict__ gin,
-             S* __restrict__ fout, S* __restrict__ gout, DevStatus* __restrict__ status,
-             int rows) {
+__device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& K,
+                                            const S* __restrict__ fin, const S* __restrict__ gin,
+                                            S* __restrict__ fout, S* __restrict__ gout, int strip,
+                                            int y0, int y1, unsigned char* shared, uint64_t* bars,
+                                            float* s_wall, int* timeout) {
   using Io = PairIo<S>;
   constexpr bool COMP = sizeof(S) == 4;
   constexpr int NST = Io::STAGES, SEG = Io::SEG, W = kMarchStrip;
-  extern __shared__ __align__(128) unsigned char march_shared[];
-  __shared__ __align__(8) uint64_t s_bar[NST];
-  __shared__ float s_wall[12];  // cavity: the side walls' links in row i
-  S* const stage0 = reinterpret_cast<S*>(march_shared);
+  S* const stage0 = reinterpret_cast<S*>(shared);
   // values handed on: [6][64] e_y = 0 of row i - 1 (lattice * 3 + k: directions 0,
   // 1, 3), [2][6][64] e_y = +1 (2, 5, 6) of rows i - 1 and i - 2 by the row's
   // parity; with walls [6][64] e_y = -1 (4, 7, 8) of row i - 1
   S* const E = stage0 + NST * 18 * SEG + 2 * threadIdx.x;
   S* const U = E + 6 * 64;
   S* const D = U + 12 * 64 + 16 / sizeof(S);
-  if (status->diverged) return;
   const int lane = threadIdx.x;
   const int nx = P.nx, ny = P.ny;
-  const int xs = blockIdx.x * W, xe = min(xs + W, nx);
-  const int xa = xs - kMarchHalo + 2 * lane;  // this lane's columns: xa, xa + 1
-  // the strip's columns, one more on each side and those they pull from are inside the lattice
-  const bool left = xs == 0, right = xs + W + 2 > nx, inside = !left && !right;
+  // the strip's 64 columns from xl; its own are [xs, xe).  A cavity has no columns
+  // beyond its walls, so there the first strip starts at the wall and the last
+  // one ends at it.
+  const int xl = BC == BC_CAVITY ? strip * W : strip * W - 2;
+  const int xs = BC == BC_CAVITY && strip == 0 ? 0 : xl + 2;
+  const bool left = strip == 0;
+  const bool right = BC == BC_CAVITY ? xl + 64 >= nx : xl + 64 > nx;
+  const int xe = BC == BC_CAVITY ? (right ? nx : xl + 62) : min(xs + W, nx);
+  const bool inside = !left && !right;  // nothing of it is at an edge of the lattice
+  const int xa = xl + 2 * lane;         // this lane's columns: xa, xa + 1
   // the staged segment (from a 16-byte boundary), cut to the row
-  const int seg0 = (xs - kMarchHalo) & ~(Io::ALIGN - 1);  // (-2 -> -4 or -8)
+  const int seg0 = (xl - 1) & ~(Io::ALIGN - 1);  // (may be negative)
   const int segb = max(seg0, 0), sege = min(seg0 + SEG, P.pitch);
   const uint32_t seg = (uint32_t)(sege - segb) * (uint32_t)sizeof(S);
-  const int y0 = blockIdx.y * rows, y1 = min(y0 + rows, ny);
-  const uint32_t bar0 = shared_addr(s_bar);
+  const uint32_t bar0 = shared_addr(bars);
   if (lane < NST)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * lane) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -264,7 +271,7 @@ __global__ void __launch_bounds__(32, sizeof(S) == 4 && BC != BC_PERIODIC ? 12 :
           break;
         }
         if (!inside) put_edge(st);
-        const S* const s = stage0 + st * 18 * SEG + (xs - kMarchHalo - seg0) + 2 * lane;
+        const S* const s = stage0 + st * 18 * SEG + (xl - seg0) + 2 * lane;
 #pragma unroll
         for (int l = 0; l < 2; ++l) {
           F2* d = l ? dg : df;
@@ -426,8 +433,22 @@ __global__ void __launch_bounds__(32, sizeof(S) == 4 && BC != BC_PERIODIC ? 12 :
         phase ^= 1;
       }
     }
-    if (lane == 0) status->timeout = 1;
+    if (lane == 0) *timeout = 1;
   }
+}
+
+template <typename S, int BC>
+__global__ void __launch_bounds__(32, kMarchWarps<S, BC>)
+    k_march2(LbParams P, PairConst K, const S* __restrict__ fin, const S* __restrict__ gin,
+             S* __restrict__ fout, S* __restrict__ gout, DevStatus* __restrict__ status,
+             int rows) {
+  extern __shared__ __align__(128) unsigned char march_shared[];
+  __shared__ __align__(8) uint64_t s_bar[PairIo<S>::STAGES];
+  __shared__ float s_wall[12];  // cavity: the side walls' links in row i
+  if (status->diverged) return;
+  const int y0 = blockIdx.y * rows;
+  march_strip<S, BC>(P, K, fin, gin, fout, gout, blockIdx.x, y0, min(y0 + rows, P.ny), march_shared,
+                     s_bar, s_wall, &status->timeout);
 }
 
 namespace march {
@@ -435,7 +456,7 @@ namespace march {
 template <typename S, int BC>
 cudaError_t go(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                DevStatus* st, int rows) {
-  const dim3 g((L.P.nx + kMarchStrip - 1) / kMarchStrip, (L.P.ny + rows - 1) / rows);
+  const dim3 g(march_strips(BC, L.P.nx), (L.P.ny + rows - 1) / rows);
   k_march2<S, BC><<<g, 32, march_smem<S>(BC), L.stream>>>(
       L.P, make_pair_const(L.P), (const S*)fin, (const S*)gin, (S*)fout, (S*)gout, st, rows);
   return cudaGetLastError();

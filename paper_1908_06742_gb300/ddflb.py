@@ -588,8 +588,8 @@ class Batch:
 
     def set_schedule(self, schedule: int):
         """0: one persistent cooperative launch per chunk of steps (device-wide
-        barrier between steps); 1: one launch per step and tile-per-CTA, the
-        chunk captured as a graph.  Same results."""
+        barrier between steps); 1: launches of two steps (one at the residual
+        checks), the chunk captured as a graph.  Same results."""
         _check(self.lib.ddflb_batch_set_schedule(self._h, int(schedule)))
         return self
 
