@@ -239,14 +239,26 @@ cudaError_t launch_step_pair(const Launch& L, const void* fin, const void* gin, 
 // periodic 16-bit lattices with nx a multiple of 4: four nodes per thread
 bool quad_step_eligible(const Launch& L);
 cudaError_t launch_step_quad(const Launch& L, const void* fin, const void* gin, void* fout,
-                             void* gout, const DevStatus* st);
+                             void* gout, const DevStatus* st, bool down);
 }  // namespace ddflb
 
 namespace {
 cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void* fout, void* gout) {
+  const bool whole = c->L.P.y0 == 0 && c->L.P.y1 == c->L.P.ny;
+  const int64_t nodes = (int64_t)c->L.P.nx * c->L.P.ny;
+  const bool half = c->L.storage != 0;
+  // steps alternate their direction where the two buffers do not fit L2 together
+  const bool down = 2 * c->lay.pops_bytes > (size_t)80 << 20 && fin == c->pops[1];
+  const bool quad = quad_step_eligible(c->L);
+  // two nodes per thread in packed arithmetic, where there are enough warps of them
+  // (16-bit periodic lattices: until the four-node kernel's wider accesses pay;
+  // 1024^2 11.65 us per step against 12.0, 700^2 7.65 against 6.8)
+  if (c->path == 0 && whole && !c->L.force && c->L.P.smodel < 2 &&
+      (half ? !(quad && c->L.P_bc == BC_PERIODIC && nodes > 900000) : nodes >= 200000))
+    return launch_step_duo(c->L, fin, gin, fout, gout, c->status, down);
   // 16-bit storage steps node groups by default (wider accesses; bit-identical)
-  if ((c->path == 3 || c->path == 0) && quad_step_eligible(c->L))
-    return launch_step_quad(c->L, fin, gin, fout, gout, c->status);
+  if ((c->path == 3 || c->path == 0) && quad)
+    return launch_step_quad(c->L, fin, gin, fout, gout, c->status, c->path == 0 && down);
   // (with walls the paired kernel is no faster than one node per thread)
   const bool pair = c->path == 2 || c->path == 3 ||
                     (c->path == 0 && c->L.storage != 0 && c->L.P_bc == BC_PERIODIC);
@@ -255,17 +267,25 @@ cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void*
   return launch_step(c->L, fin, gin, fout, gout, c->status);
 }
 
+// Smallest lattice that takes two steps per launch: below it strips of enough rows
+// do not fill the GPU.  us per step, two per launch against the best single-step
+// kernel: FP32 periodic 1100^2 26.7 / 25.4, 1200^2 28.6 / 29.1, 2048^2 68 / 84;
+// FP32 cavity 1200^2 31.5 / 29.5, 1400^2 39.3 / 39.9; 16-bit cavity 2048^2 58.5 /
+// 56.1, 4096^2 210 / 246; 16-bit periodic 2048^2 54.3 / 49.3 (four nodes per
+// thread), 4096^2 180 / 186.
+int64_t march_min_nodes(const Launch& L) {
+  if (L.storage == 0) return L.P_bc == BC_PERIODIC ? 1400000 : 2000000;
+  return quad_step_eligible(L) && L.P_bc == BC_PERIODIC ? 10000000 : 6000000;
+}
+
 // Rows per warp of the two-step kernel (ddflb_march.cuh), or 0 where steps go
 // one per launch: the y-slab contexts, forced lattices and central-moment
 // scalar models (whose collisions have no packed form), an explicit path, and
-// lattices too small to fill the GPU with strips of enough rows.  Measured, two
-// steps per launch against the one-step kernels (us per step): FP32 1024^2 26
-// against 24.4, 2048^2 74 against 91.5; 16-bit 2048^2 cavity 59 against 65.5,
-// 1023 x 767 16.5 against 12.6.
+// lattices too small.
 int choose_march_rows(const ddflb_ctx* c) {
   const LbParams& P = c->L.P;
   if (c->path != 0 || P.y0 != 0 || P.y1 != P.ny || c->L.force || P.smodel >= 2) return 0;
-  if ((int64_t)P.nx * P.ny < kMarchMinNodes) return 0;
+  if ((int64_t)P.nx * P.ny < march_min_nodes(c->L)) return 0;
   // strips x chunks in waves of 15 warps an SM, plus most of a chunk at the end
   // while the last ones finish (FP32 8192^2, rows 16 / 32 / 64 / 128: 878, 853,
   // 870, 1023 us per step; 4096^2: 231, 237, 261, 325)

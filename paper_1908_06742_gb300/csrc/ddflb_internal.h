@@ -14,7 +14,6 @@ inline int march_strips(int bc, int nx) {
   if (bc == BC_CAVITY) return nx <= 64 ? 1 : 1 + (nx - 64 + kMarchStrip - 1) / kMarchStrip;
   return (nx + kMarchStrip - 1) / kMarchStrip;
 }
-constexpr int64_t kMarchMinNodes = (int64_t)1 << 21;  // smallest lattice it is used for
 constexpr int kReduceThreads = 256;
 constexpr int kReduceBlocks = 608;  // 4 per SM on a 152-SM GB300; fixed for deterministic sums
 
@@ -59,6 +58,9 @@ cudaError_t launch_halo_local(const HaloSlabs& H, int storage, cudaStream_t stre
 
 cudaError_t launch_step(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                         const DevStatus* st);
+// one step, two nodes per thread, packed arithmetic (ddflb_step_duo.cu)
+cudaError_t launch_step_duo(const Launch& L, const void* fin, const void* gin, void* fout,
+                            void* gout, const DevStatus* st, bool down);
 // two time steps in one launch (ddflb_march.cuh); rows: lattice rows per CTA
 cudaError_t launch_march2_f32(const Launch& L, const void* fin, const void* gin, void* fout,
                               void* gout, DevStatus* st, int rows);

@@ -28,25 +28,6 @@ template <> struct PairIo<float> {
   static __device__ __forceinline__ F2 round(F2 v) { return v; }
 };
 
-template <typename S> __device__ __forceinline__ F2 widen(unsigned w);
-template <> __device__ __forceinline__ F2 widen<__half>(unsigned w) {
-  return __half22float2(*reinterpret_cast<const __half2*>(&w));
-}
-template <> __device__ __forceinline__ F2 widen<__nv_bfloat16>(unsigned w) {
-  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
-__device__ __forceinline__ float widen1(__half v) { return __half2float(v); }
-__device__ __forceinline__ float widen1(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <typename S> __device__ __forceinline__ unsigned narrow(F2 v);
-template <> __device__ __forceinline__ unsigned narrow<__half>(F2 v) {
-  const __half2 h = __floats2half2_rn(v.x, v.y);
-  return *reinterpret_cast<const unsigned*>(&h);
-}
-template <> __device__ __forceinline__ unsigned narrow<__nv_bfloat16>(F2 v) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
-  return *reinterpret_cast<const unsigned*>(&h);
-}
-
 template <typename S> struct PairIo {
   static constexpr int ALIGN = 8, SEG = 72, STAGES = 3;
   static __device__ __forceinline__ F2 ld(const S* p) {
@@ -104,7 +85,7 @@ template <typename S>
 constexpr size_t march_smem(int bc) {
   // the staged rows, three rows of values handed on (6 planes each) and, with
   // walls, the e_y = -1 values of one row
-  return (size_t)(PairIo<S>::STAGES * 18 * PairIo<S>::SEG + 18 * 64) * sizeof(S) + 16 +
+  return (size_t)(PairIo<S>::STAGES * 18 * PairIo<S>::SEG + 18 * 64) * sizeof(S) +
          (bc != BC_PERIODIC ? 6 * 64 * sizeof(S) : 0);
 }
 
@@ -140,12 +121,16 @@ __device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& 
   constexpr bool COMP = sizeof(S) == 4;
   constexpr int NST = Io::STAGES, SEG = Io::SEG, W = kMarchStrip;
   S* const stage0 = reinterpret_cast<S*>(shared);
+  // stage 0, the values handed on, the other stages, D: the outer lanes' reads one
+  // element beside the handed-on planes stay inside (and without margins 15
+  // periodic FP32 warps fit an SM)
+  auto stage_at = [&](int k) { return stage0 + k * 18 * SEG + (k > 0 ? 18 * 64 : 0); };
   // values handed on: [6][64] e_y = 0 of row i - 1 (lattice * 3 + k: directions 0,
   // 1, 3), [2][6][64] e_y = +1 (2, 5, 6) of rows i - 1 and i - 2 by the row's
   // parity; with walls [6][64] e_y = -1 (4, 7, 8) of row i - 1
-  S* const E = stage0 + NST * 18 * SEG + 2 * threadIdx.x;
+  S* const E = stage0 + 18 * SEG + 2 * threadIdx.x;
   S* const U = E + 6 * 64;
-  S* const D = U + 12 * 64 + 16 / sizeof(S);
+  S* const D = stage0 + NST * 18 * SEG + 18 * 64 + 2 * threadIdx.x;
   const int lane = threadIdx.x;
   const int nx = P.nx, ny = P.ny;
   // the strip's 64 columns from xl; its own are [xs, xe).  A cavity has no columns
@@ -190,7 +175,7 @@ __device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& 
       }
       asm volatile(
           "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
-          "[%3];" ::"r"(pdst + (uint32_t)(st * 18 * SEG * (int)sizeof(S))),
+          "[%3];" ::"r"(pdst + (uint32_t)((st * 18 * SEG + (st > 0 ? 18 * 64 : 0)) * (int)sizeof(S))),
           "l"(psrc + (int64_t)y * P.pitch), "r"(seg), "r"(bar)
           : "memory");
     }
@@ -242,7 +227,7 @@ __device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& 
       for (int j = 0; j < NEDGE; ++j) {
         const int e = lane + 32 * j, side = e / 36, p = e % 36 >> 1, c = e & 1;
         if (e < 72 && (side ? right : left))
-          stage0[(st * 18 + p) * SEG + (side ? nx + c : c - 2) - seg0] = edge[j];
+          stage_at(st)[p * SEG + (side ? nx + c : c - 2) - seg0] = edge[j];
       }
       // (the next copy into this stage goes through the async proxy)
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -271,7 +256,7 @@ __device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& 
           break;
         }
         if (!inside) put_edge(st);
-        const S* const s = stage0 + st * 18 * SEG + (xl - seg0) + 2 * lane;
+        const S* const s = stage_at(st) + (xl - seg0) + 2 * lane;
 #pragma unroll
         for (int l = 0; l < 2; ++l) {
           F2* d = l ? dg : df;

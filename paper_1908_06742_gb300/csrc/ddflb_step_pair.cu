@@ -206,12 +206,14 @@ template <typename S, int BC>
 __global__ void __maxnreg__(96) k_step_quad(LbParams P, const S* __restrict__ fin,
                                                    const S* __restrict__ gin,
                                                    S* __restrict__ fout, S* __restrict__ gout,
-                                                   const DevStatus* __restrict__ status) {
+                                                   const DevStatus* __restrict__ status,
+                                                   bool down) {
   constexpr int EX[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
   constexpr int EY[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
   const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  if (x0 >= P.nx || y >= P.ny) return;
+  // down: rows in descending order (as k_step_duo)
+  const int yb = blockIdx.y * blockDim.y + threadIdx.y, y = down ? P.ny - 1 - yb : yb;
+  if (x0 >= P.nx || yb >= P.ny) return;
   if (status != nullptr && status->diverged) return;
   const int nx = P.nx, ny = P.ny;
   const int64_t pl = P.plane;
@@ -318,28 +320,28 @@ bool quad_step_eligible(const Launch& L) {
 namespace {
 template <typename S, int BC>
 cudaError_t go_quad(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
-                    const DevStatus* st) {
+                    const DevStatus* st, bool down) {
   const dim3 b(128, 1);
   const dim3 g((L.P.nx / 4 + b.x - 1) / b.x, L.P.ny);
   k_step_quad<S, BC><<<g, b, 0, L.stream>>>(L.P, (const S*)fin, (const S*)gin, (S*)fout,
-                                            (S*)gout, st);
+                                            (S*)gout, st, down);
   return cudaGetLastError();
 }
 template <typename S>
 cudaError_t go_quad_bc(const Launch& L, const void* fin, const void* gin, void* fout,
-                       void* gout, const DevStatus* st) {
+                       void* gout, const DevStatus* st, bool down) {
   switch (L.P_bc) {
-    case BC_PERIODIC: return go_quad<S, BC_PERIODIC>(L, fin, gin, fout, gout, st);
-    case BC_CAVITY: return go_quad<S, BC_CAVITY>(L, fin, gin, fout, gout, st);
-    default: return go_quad<S, BC_CHANNEL>(L, fin, gin, fout, gout, st);
+    case BC_PERIODIC: return go_quad<S, BC_PERIODIC>(L, fin, gin, fout, gout, st, down);
+    case BC_CAVITY: return go_quad<S, BC_CAVITY>(L, fin, gin, fout, gout, st, down);
+    default: return go_quad<S, BC_CHANNEL>(L, fin, gin, fout, gout, st, down);
   }
 }
 }  // namespace
 
 cudaError_t launch_step_quad(const Launch& L, const void* fin, const void* gin, void* fout,
-                             void* gout, const DevStatus* st) {
-  if (L.storage == 1) return go_quad_bc<__half>(L, fin, gin, fout, gout, st);
-  return go_quad_bc<__nv_bfloat16>(L, fin, gin, fout, gout, st);
+                             void* gout, const DevStatus* st, bool down) {
+  if (L.storage == 1) return go_quad_bc<__half>(L, fin, gin, fout, gout, st, down);
+  return go_quad_bc<__nv_bfloat16>(L, fin, gin, fout, gout, st, down);
 }
 
 bool pair_step_eligible(const Launch& L) {

@@ -6,7 +6,8 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
-NODES = 1 << 21  # the smallest lattice that takes two steps per launch
+# lattices large enough to take two steps per launch, by storage
+NODES = {"fp32": 1 << 21, "fp16": 10_100_000, "bf16": 10_100_000}
 
 
 def _fields(torch, nx, ny, seed):
@@ -27,24 +28,24 @@ def _same(torch, a, b):
                for x, y in zip(a, b))
 
 
-SHAPES = [(40, 52500), (59, None), (60, None), (61, None), (62, None), (119, None), (121, None),
-          (122, None), (190, None), (1 << 20, 2), (700001, 3), (300003, 7), (1025, 2049)]
+WIDTHS = {"fp32": (40, 59, 60, 61, 62, 119, 121, 122, 190), "fp16": (179, 180, 181, 182, 242),
+          "bf16": (239, 240, 241, 245)}
+HEIGHTS = (2, 3, 7, 2049)
 
 
-@pytest.mark.parametrize("storage", ["fp32", "fp16", "bf16"])
 @pytest.mark.parametrize("bc", ["periodic", "cavity", "channel"])
-@pytest.mark.parametrize("nx,ny", SHAPES)
+@pytest.mark.parametrize("storage,nx,ny", [(s, w, -(-NODES[s] // w)) for s in WIDTHS
+                                           for w in WIDTHS[s]]
+                         + [(s, NODES[s] // h + 1, h) for s in WIDTHS for h in HEIGHTS])
 def test_two_steps_match_single_steps(bc, storage, nx, ny):
     import torch
     from paper_1908_06742_gb300 import ddflb as D
-    ny = ny or -(-NODES // nx)
     cfg = D.Config(nx=nx, ny=ny, bc=bc, storage=storage, nu=0.02, diffusivity=0.03, u_lid=0.08,
                    phi_lid=1.2, phi_wall=0.4)
     f = _fields(torch, nx, ny, nx + ny)
-    # two launches of two steps, one single step, then 64 steps as a graph
-    assert _same(torch, _run(D, cfg, f, 0, (5,)), _run(D, cfg, f, 1, (5,)))
-    if nx in (61, 121, 1025):
-        assert _same(torch, _run(D, cfg, f, 0, (67,)), _run(D, cfg, f, 1, (67,)))
+    # two launches of two steps, one single step; at a few sizes also a graph of 64
+    for steps in ((5,), (67,)) if nx in (61, 121, 181, 241) else ((5,),):
+        assert _same(torch, _run(D, cfg, f, 0, steps), _run(D, cfg, f, 1, steps))
 
 
 @pytest.mark.parametrize("storage", ["fp32", "fp16"])
@@ -53,8 +54,8 @@ def test_checks_and_srt(storage):
     the SRT collision runs through the same kernel."""
     import torch
     from paper_1908_06742_gb300 import ddflb as D
-    cfg = D.Config(nx=1537, ny=1400, storage=storage, scalar_model="srt", check_every=3)
-    f = _fields(torch, 1537, 1400, 9)
+    cfg = D.Config(nx=1537, ny=NODES[storage] // 1537 + 1, storage=storage, scalar_model="srt", check_every=3)
+    f = _fields(torch, cfg.nx, cfg.ny, 9)
     got = []
     for path in (0, 1):
         lat = D.Lattice(cfg).set_path(path).init(*f)
