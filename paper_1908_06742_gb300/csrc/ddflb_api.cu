@@ -243,19 +243,31 @@ cudaError_t launch_step_quad(const Launch& L, const void* fin, const void* gin, 
 }  // namespace ddflb
 
 namespace {
+// Smallest lattice that steps two nodes per thread in packed arithmetic: below it
+// one node per thread has more warps to hide latency with.  us per step, one node
+// -> two: FP32 cascaded 256^2 3.08 -> 3.10, 300^2 3.95 -> 3.66; BF16 96^2 1.98 ->
+// 2.19, 160^2 2.50 -> 2.40.
+int64_t duo_min_nodes(const Launch& L) {
+  if (L.storage == 0) return 85000;
+  return L.force || L.P.smodel >= 2 ? 20000 : 0;
+}
+
 cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void* fout, void* gout) {
   const bool whole = c->L.P.y0 == 0 && c->L.P.y1 == c->L.P.ny;
   const int64_t nodes = (int64_t)c->L.P.nx * c->L.P.ny;
-  const bool half = c->L.storage != 0;
   // steps alternate their direction where the two buffers do not fit L2 together
   const bool down = 2 * c->lay.pops_bytes > (size_t)80 << 20 && fin == c->pops[1];
   const bool quad = quad_step_eligible(c->L);
-  // two nodes per thread in packed arithmetic, where there are enough warps of them
-  // (16-bit periodic lattices: until the four-node kernel's wider accesses pay;
-  // 1024^2 11.65 us per step against 12.0, 700^2 7.65 against 6.8)
-  if (c->path == 0 && whole && !c->L.force && c->L.P.smodel < 2 &&
-      (half ? !(quad && c->L.P_bc == BC_PERIODIC && nodes > 900000) : nodes >= 200000))
-    return launch_step_duo(c->L, fin, gin, fout, gout, c->status, down);
+  // two nodes per thread in packed arithmetic (unforced MRT 16-bit periodic lattices:
+  // until the four-node kernel's wider accesses pay; 1024^2 11.65 us per step
+  // against 12.0, 700^2 7.65 against 6.8)
+  if (c->path == 0 && whole && nodes >= duo_min_nodes(c->L) &&
+      !(quad && c->L.P_bc == BC_PERIODIC && nodes > 900000)) {
+    auto* launch = c->L.storage == 0   ? launch_step_duo_f32
+                   : c->L.storage == 1 ? launch_step_duo_f16
+                                       : launch_step_duo_bf16;
+    return launch(c->L, fin, gin, fout, gout, c->status, down);
+  }
   // 16-bit storage steps node groups by default (wider accesses; bit-identical)
   if ((c->path == 3 || c->path == 0) && quad)
     return launch_step_quad(c->L, fin, gin, fout, gout, c->status, c->path == 0 && down);

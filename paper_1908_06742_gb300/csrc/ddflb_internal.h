@@ -58,9 +58,14 @@ cudaError_t launch_halo_local(const HaloSlabs& H, int storage, cudaStream_t stre
 
 cudaError_t launch_step(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                         const DevStatus* st);
-// one step, two nodes per thread, packed arithmetic (ddflb_step_duo.cu)
-cudaError_t launch_step_duo(const Launch& L, const void* fin, const void* gin, void* fout,
-                            void* gout, const DevStatus* st, bool down);
+// one step, two nodes per thread, packed arithmetic (ddflb_step_duo.cuh); down:
+// the rows in descending order
+cudaError_t launch_step_duo_f32(const Launch& L, const void* fin, const void* gin, void* fout,
+                                void* gout, const DevStatus* st, bool down);
+cudaError_t launch_step_duo_f16(const Launch& L, const void* fin, const void* gin, void* fout,
+                                void* gout, const DevStatus* st, bool down);
+cudaError_t launch_step_duo_bf16(const Launch& L, const void* fin, const void* gin, void* fout,
+                                 void* gout, const DevStatus* st, bool down);
 // two time steps in one launch (ddflb_march.cuh); rows: lattice rows per CTA
 cudaError_t launch_march2_f32(const Launch& L, const void* fin, const void* gin, void* fout,
                               void* gout, DevStatus* st, int rows);
