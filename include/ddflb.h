@@ -299,11 +299,11 @@ ddflb_status ddflb_set_block(ddflb_ctx* c, int32_t block_x, int32_t block_y);
  * 3 four adjacent nodes per thread with aligned 8-byte accesses (as 2, with
  * nx a multiple of 4; nodes next to a wall one by one; otherwise falls back to
  * 2, then 1);
- * 0 (default) = by size, for unforced lattices with MRT or SRT scalar: four
- * steps per launch on small ones (about 256^2 at most; also with a steady force),
- * two on large ones (from 1.4 to 10 million nodes on), single steps with two
- * nodes per thread between them and where a call or a residual check leaves
- * some; else as 1, or 2 and 3 for 16-bit storage.  All give bit-identical
+ * 0 (default) = by size: four steps per launch on small lattices (about 256^2
+ * at most, no time-dependent force), two on large ones (unforced MRT or SRT
+ * scalar, from 1.4 to 10 million nodes on), single steps with two nodes per
+ * thread between them and where a call or a residual check leaves some (16-bit
+ * periodic ones of a million nodes with four).  All give bit-identical
  * results; which is faster depends on the shape, so the autotuner times them. */
 ddflb_status ddflb_set_path(ddflb_ctx* c, int32_t path);
 

@@ -271,9 +271,7 @@ cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void*
   // 16-bit storage steps node groups by default (wider accesses; bit-identical)
   if ((c->path == 3 || c->path == 0) && quad)
     return launch_step_quad(c->L, fin, gin, fout, gout, c->status, c->path == 0 && down);
-  // (with walls the paired kernel is no faster than one node per thread)
-  const bool pair = c->path == 2 || c->path == 3 ||
-                    (c->path == 0 && c->L.storage != 0 && c->L.P_bc == BC_PERIODIC);
+  const bool pair = c->path == 2 || c->path == 3;
   if (pair && pair_step_eligible(c->L))
     return launch_step_pair(c->L, fin, gin, fout, gout, c->status);
   return launch_step(c->L, fin, gin, fout, gout, c->status);
@@ -334,8 +332,7 @@ cudaError_t run_two(const ddflb_ctx* c, int src) {
 // (384^2: 4.1 us per step, two or four steps per launch 4.3).
 int choose_tile(const ddflb_ctx* c) {
   const LbParams& P = c->L.P;
-  if (c->path != 0 || P.y0 != 0 || P.y1 != P.ny || c->p.force_omega != 0.0 || P.smodel >= 2)
-    return -1;
+  if (c->path != 0 || P.y0 != 0 || P.y1 != P.ny || c->p.force_omega != 0.0) return -1;
   if (P.nx < kTileSteps || P.ny < kTileSteps) return -1;  // (a region wraps once at most)
   for (int k = 0; k < kTileShapes; ++k) {
     const int tx = kTileShape[k][0], ty = kTileShape[k][1];
@@ -349,10 +346,12 @@ cudaError_t run_tile(const ddflb_ctx* c, int src) {
   const size_t gofs = c->lay.gofs;
   const char* fi = (const char*)c->pops[src];
   char* fo = (char*)c->pops[src ^ 1];
-  auto* launch = c->L.storage == 0   ? launch_tile_f32
-                 : c->L.storage == 1 ? launch_tile_f16
-                                     : launch_tile_bf16;
-  return launch(c->L, fi, fi + gofs, fo, fo + gofs, c->status, c->tile);
+  static TileLaunch* const launch[3][3] = {
+      {launch_tile_f32, launch_tile_f16, launch_tile_bf16},
+      {launch_tile_cascaded_f32, launch_tile_cascaded_f16, launch_tile_cascaded_bf16},
+      {launch_tile_central_f32, launch_tile_central_f16, launch_tile_central_bf16}};
+  const int model = c->L.P.smodel < 2 ? 0 : c->L.P.smodel - 1;
+  return launch[model][c->L.storage](c->L, fi, fi + gofs, fo, fo + gofs, c->status, c->tile);
 }
 
 // Small lattices are launch-bound: runs of kGraphSteps steps between checks

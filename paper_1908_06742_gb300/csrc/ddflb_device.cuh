@@ -417,25 +417,38 @@ __device__ __forceinline__ void relax_source(const float w[9], const Neq& n, con
 // shift by u.  The raw image of the central equilibria equals the raw
 // equilibria of Eq. (eqmrawmoment_CDE) up to third order; in the fourth-order
 // moment it is larger by 2 c phi ((b2 - 1) ux^2 + (b1 - 1) uy^2).
+// (Products are fused into sums by hand here and below, so that every kernel
+// rounds alike: the compiler's own choice depends on what surrounds the code.)
 struct CNeq {
   float x, y, xx, yy, xy, xxy, xyy, xxyy;
 };
 
 __device__ __forceinline__ CNeq central_neq(const LbParams& P, const Neq& n, const Macro& q) {
   const float c = 1.0f / 3.0f, ux = q.ux, uy = q.uy;
-  const float rx = n.n1, ry = n.n2, rxx = 0.5f * (n.n3 + n.n4), ryy = 0.5f * (n.n3 - n.n4);
+  const float rx = n.n1, ry = n.n2;
+  const float rxx = __fmul_rn(0.5f, __fadd_rn(n.n3, n.n4));
+  const float ryy = __fmul_rn(0.5f, __fsub_rn(n.n3, n.n4));
   const float rxy = n.n5, rxxy = n.n6, rxyy = n.n7;
-  const float rxxyy = n.n8 - 2.0f * c * q.phi * ((P.b2 - 1.0f) * ux * ux + (P.b1 - 1.0f) * uy * uy);
+  const float ux2 = 2.0f * ux, uy2 = 2.0f * uy, uxx = __fmul_rn(ux, ux), uyy = __fmul_rn(uy, uy);
+  const float p2 = __fmul_rn(ux2, uy), p4 = __fmul_rn(4.0f * ux, uy);
+  // b2 - 1 and b1 - 1 times the squares
+  const float in = __fmaf_rn(__fmul_rn(__fsub_rn(P.b2, 1.0f), ux), ux,
+                             __fmul_rn(__fmul_rn(__fsub_rn(P.b1, 1.0f), uy), uy));
   CNeq v;
   v.x = rx;
   v.y = ry;
-  v.xx = rxx - 2.0f * ux * rx;
-  v.yy = ryy - 2.0f * uy * ry;
-  v.xy = rxy - uy * rx - ux * ry;
-  v.xxy = rxxy - 2.0f * ux * rxy + ux * ux * ry - uy * rxx + 2.0f * ux * uy * rx;
-  v.xyy = rxyy - 2.0f * uy * rxy + uy * uy * rx - ux * ryy + 2.0f * ux * uy * ry;
-  v.xxyy = rxxyy - 2.0f * ux * rxyy - 2.0f * uy * rxxy + ux * ux * ryy + uy * uy * rxx +
-           4.0f * ux * uy * rxy - 2.0f * ux * ux * uy * ry - 2.0f * ux * uy * uy * rx;
+  v.xx = __fmaf_rn(-ux2, rx, rxx);
+  v.yy = __fmaf_rn(-uy2, ry, ryy);
+  v.xy = __fmaf_rn(-ux, ry, __fmaf_rn(-uy, rx, rxy));
+  v.xxy = __fmaf_rn(-ux2, rxy, rxxy);
+  v.xxy = __fmaf_rn(p2, rx, __fmaf_rn(-uy, rxx, __fmaf_rn(uxx, ry, v.xxy)));
+  v.xyy = __fmaf_rn(-uy2, rxy, rxyy);
+  v.xyy = __fmaf_rn(p2, ry, __fmaf_rn(-ux, ryy, __fmaf_rn(uyy, rx, v.xyy)));
+  float t = __fmaf_rn(-__fmul_rn(2.0f * c, q.phi), in, n.n8);  // the raw moment's change
+  t = __fmaf_rn(-uy2, rxxy, __fmaf_rn(-ux2, rxyy, t));
+  t = __fmaf_rn(p4, rxy, __fmaf_rn(uyy, rxx, __fmaf_rn(uxx, ryy, t)));
+  t = __fmaf_rn(-__fmul_rn(__fmul_rn(ux2, ux), uy), ry, t);
+  v.xxyy = __fmaf_rn(-__fmul_rn(p2, uy), rx, t);
   return v;
 }
 
@@ -445,21 +458,39 @@ __device__ __forceinline__ CNeq central_neq(const LbParams& P, const Neq& n, con
 __device__ __forceinline__ void relax_central(const float w[9], const CNeq& v, const Macro& q,
                                               float d[9]) {
   const float ux = q.ux, uy = q.uy;
-  const float Dx = -w[1] * v.x, Dy = -w[2] * v.y;
-  const float Ds = -w[3] * (v.xx + v.yy), Dd = -w[4] * (v.xx - v.yy);
-  const float Dxx = 0.5f * (Ds + Dd), Dyy = 0.5f * (Ds - Dd);
-  const float Dxy = -w[5] * v.xy, Dxxy = -w[6] * v.xxy, Dxyy = -w[7] * v.xyy;
-  const float Dxxyy = -w[8] * v.xxyy;
-  const float Rxx = Dxx + 2.0f * ux * Dx, Ryy = Dyy + 2.0f * uy * Dy;
-  const float Rxy = Dxy + uy * Dx + ux * Dy;
-  const float Rxxy = Dxxy + 2.0f * ux * Dxy + ux * ux * Dy + uy * Dxx + 2.0f * ux * uy * Dx;
-  const float Rxyy = Dxyy + 2.0f * uy * Dxy + uy * uy * Dx + ux * Dyy + 2.0f * ux * uy * Dy;
-  const float Rxxyy = Dxxyy + 2.0f * ux * Dxyy + 2.0f * uy * Dxxy + ux * ux * Dyy + uy * uy * Dxx +
-                      4.0f * ux * uy * Dxy + 2.0f * ux * ux * uy * Dy + 2.0f * ux * uy * uy * Dx;
-  float dd[9];
-  populations(0.0f, Dx, Dy, Rxx + Ryy, Rxx - Ryy, Rxy, Rxxy, Rxyy, Rxxyy, dd);
-#pragma unroll
-  for (int a = 0; a < 9; ++a) d[a] += dd[a];
+  const float Dx = __fmul_rn(-w[1], v.x), Dy = __fmul_rn(-w[2], v.y);
+  const float vs = __fadd_rn(v.xx, v.yy), vd = __fsub_rn(v.xx, v.yy);
+  const float Dd = __fmul_rn(-w[4], vd);
+  const float Dxx = __fmul_rn(0.5f, __fmaf_rn(-w[3], vs, Dd));
+  const float Dyy = __fmul_rn(0.5f, __fmaf_rn(-w[3], vs, -Dd));
+  const float Dxy = __fmul_rn(-w[5], v.xy), Dxxy = __fmul_rn(-w[6], v.xxy);
+  const float Dxyy = __fmul_rn(-w[7], v.xyy), Dxxyy = __fmul_rn(-w[8], v.xxyy);
+  const float ux2 = 2.0f * ux, uy2 = 2.0f * uy, uxx = __fmul_rn(ux, ux), uyy = __fmul_rn(uy, uy);
+  const float p2 = __fmul_rn(ux2, uy), p4 = __fmul_rn(4.0f * ux, uy);
+  const float Rxx = __fmaf_rn(ux2, Dx, Dxx), Ryy = __fmaf_rn(uy2, Dy, Dyy);
+  const float Rxy = __fmaf_rn(ux, Dy, __fmaf_rn(uy, Dx, Dxy));
+  float Rxxy = __fmaf_rn(uxx, Dy, __fmaf_rn(ux2, Dxy, Dxxy));
+  Rxxy = __fmaf_rn(p2, Dx, __fmaf_rn(uy, Dxx, Rxxy));
+  float Rxyy = __fmaf_rn(uyy, Dx, __fmaf_rn(uy2, Dxy, Dxyy));
+  Rxyy = __fmaf_rn(p2, Dy, __fmaf_rn(ux, Dyy, Rxyy));
+  float R4 = __fmaf_rn(uy2, Dxxy, __fmaf_rn(ux2, Dxyy, Dxxyy));
+  R4 = __fmaf_rn(p4, Dxy, __fmaf_rn(uyy, Dxx, __fmaf_rn(uxx, Dyy, R4)));
+  R4 = __fmaf_rn(__fmul_rn(__fmul_rn(ux2, ux), uy), Dy, R4);
+  R4 = __fmaf_rn(__fmul_rn(p2, uy), Dx, R4);
+  // the increments of populations(), whose sums have nothing to fuse
+  const float m3 = __fadd_rn(Rxx, Ryy), m4 = __fsub_rn(Rxx, Ryy);
+  const float kxx = 0.5f * __fadd_rn(m3, m4), kyy = 0.5f * __fsub_rn(m3, m4);
+  const float p = __fadd_rn(Rxy, R4), s = __fadd_rn(Rxxy, Rxyy);
+  const float r = __fsub_rn(R4, Rxy), e = __fsub_rn(Rxxy, Rxyy);
+  d[0] += __fsub_rn(R4, m3);
+  d[1] += 0.5f * __fsub_rn(__fsub_rn(__fadd_rn(Dx, kxx), Rxyy), R4);
+  d[2] += 0.5f * __fsub_rn(__fsub_rn(__fadd_rn(Dy, kyy), Rxxy), R4);
+  d[3] += 0.5f * __fsub_rn(__fadd_rn(__fsub_rn(kxx, Dx), Rxyy), R4);
+  d[4] += 0.5f * __fsub_rn(__fadd_rn(__fsub_rn(kyy, Dy), Rxxy), R4);
+  d[5] += 0.25f * __fadd_rn(p, s);
+  d[6] += 0.25f * __fadd_rn(r, e);
+  d[7] += 0.25f * __fsub_rn(p, s);
+  d[8] += 0.25f * __fsub_rn(r, e);
 }
 
 // App. C (cascaded): the changes h1..h8 in the orthogonal basis K, found order by
@@ -468,24 +499,35 @@ __device__ __forceinline__ void relax_central(const float w[9], const CNeq& v, c
 // the paper's inner products and expansion of g~ require).
 __device__ __forceinline__ void relax_cascaded(const float w[9], const CNeq& v, const Macro& q,
                                                float d[9]) {
-  const float ux = q.ux, uy = q.uy, ux2 = ux * ux, uy2 = uy * uy;
-  const float h1 = -w[1] * v.x * (1.0f / 6.0f);
-  const float h2 = -w[2] * v.y * (1.0f / 6.0f);
-  const float h3 = -w[3] * (v.xx + v.yy) * (1.0f / 12.0f) + (ux * h1 + uy * h2);
-  const float h4 = -w[4] * (v.xx - v.yy) * 0.25f + 3.0f * (ux * h1 - uy * h2);
-  const float h5 = -w[5] * v.xy * 0.25f + 1.5f * (ux * h2 + uy * h1);
-  const float h6 = w[6] * v.xxy * 0.25f - 2.0f * ux * h5 - 0.5f * uy * h4 - 1.5f * uy * h3 +
-                   (1.0f + 1.5f * ux2) * h2 + 3.0f * ux * uy * h1;
-  const float h7 = w[7] * v.xyy * 0.25f - 2.0f * uy * h5 + 0.5f * ux * h4 - 1.5f * ux * h3 +
-                   3.0f * ux * uy * h2 + (1.0f + 1.5f * uy2) * h1;
-  const float h8 = -w[8] * v.xxyy * 0.25f - 2.0f * ux * h7 - 2.0f * uy * h6 -
-                   4.0f * ux * uy * h5 + 0.5f * (ux2 - uy2) * h4 -
-                   (2.0f + 1.5f * (ux2 + uy2)) * h3 + (2.0f + 3.0f * ux2) * uy * h2 +
-                   (2.0f + 3.0f * uy2) * ux * h1;
+  const float ux = q.ux, uy = q.uy, uxx = __fmul_rn(ux, ux), uyy = __fmul_rn(uy, uy);
+  const float ux2 = 2.0f * ux, uy2 = 2.0f * uy;
+  const float p3 = __fmul_rn(__fmul_rn(3.0f, ux), uy), p4 = __fmul_rn(4.0f * ux, uy);
+  const float vs = __fadd_rn(v.xx, v.yy), vd = __fsub_rn(v.xx, v.yy);
+  const float h1 = __fmul_rn(__fmul_rn(-w[1], v.x), 1.0f / 6.0f);
+  const float h2 = __fmul_rn(__fmul_rn(-w[2], v.y), 1.0f / 6.0f);
+  const float t2 = __fmul_rn(uy, h2);
+  const float h3 = __fmaf_rn(__fmul_rn(-w[3], vs), 1.0f / 12.0f, __fmaf_rn(ux, h1, t2));
+  const float h4 = __fmaf_rn(3.0f, __fmaf_rn(ux, h1, -t2), 0.25f * __fmul_rn(-w[4], vd));
+  const float h5 = __fmaf_rn(1.5f, __fmaf_rn(uy, h1, __fmul_rn(ux, h2)),
+                             0.25f * __fmul_rn(-w[5], v.xy));
+  float t = __fmaf_rn(__fmul_rn(w[6], v.xxy), 0.25f, -__fmul_rn(ux2, h5));
+  t = __fmaf_rn(-__fmul_rn(1.5f, uy), h3, __fmaf_rn(-0.5f * uy, h4, t));
+  t = __fmaf_rn(__fmaf_rn(1.5f, uxx, 1.0f), h2, t);
+  const float h6 = __fmaf_rn(p3, h1, t);
+  t = __fmaf_rn(__fmul_rn(w[7], v.xyy), 0.25f, -__fmul_rn(uy2, h5));
+  t = __fmaf_rn(-__fmul_rn(1.5f, ux), h3, __fmaf_rn(0.5f * ux, h4, t));
+  t = __fmaf_rn(p3, h2, t);
+  const float h7 = __fmaf_rn(__fmaf_rn(1.5f, uyy, 1.0f), h1, t);
+  t = __fmaf_rn(__fmul_rn(-w[8], v.xxyy), 0.25f, -__fmul_rn(ux2, h7));
+  t = __fmaf_rn(-p4, h5, __fmaf_rn(-uy2, h6, t));
+  t = __fmaf_rn(0.5f * __fsub_rn(uxx, uyy), h4, t);
+  t = __fmaf_rn(-__fmaf_rn(1.5f, __fadd_rn(uxx, uyy), 2.0f), h3, t);
+  t = __fmaf_rn(__fmul_rn(__fmaf_rn(3.0f, uxx, 2.0f), uy), h2, t);
+  const float h8 = __fmaf_rn(__fmul_rn(__fmaf_rn(3.0f, uyy, 2.0f), ux), h1, t);
   constexpr int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
   constexpr int ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
 #pragma unroll
-  for (int a = 0; a < 9; ++a) {
+  for (int a = 0; a < 9; ++a) {  // (the coefficients are 0 or powers of two: nothing to fuse)
     const float x = (float)ex[a], y = (float)ey[a], x2 = x * x, y2 = y * y;
     d[a] += x * h1 + y * h2 + (3.0f * (x2 + y2) - 4.0f) * h3 + (x2 - y2) * h4 + x * y * h5 +
             (2.0f * y - 3.0f * x2 * y) * h6 + (2.0f * x - 3.0f * x * y2) * h7 +

@@ -77,12 +77,11 @@ cudaError_t launch_march2_bf16(const Launch& L, const void* fin, const void* gin
 // shapes it is built for, smallest first
 constexpr int kTileSteps = 4, kTileShapes = 5;
 constexpr int kTileShape[kTileShapes][2] = {{8, 4}, {8, 8}, {16, 8}, {16, 16}, {32, 14}};
-cudaError_t launch_tile_f32(const Launch& L, const void* fin, const void* gin, void* fout,
-                            void* gout, const DevStatus* st, int shape);
-cudaError_t launch_tile_f16(const Launch& L, const void* fin, const void* gin, void* fout,
-                            void* gout, const DevStatus* st, int shape);
-cudaError_t launch_tile_bf16(const Launch& L, const void* fin, const void* gin, void* fout,
-                             void* gout, const DevStatus* st, int shape);
+typedef cudaError_t TileLaunch(const Launch& L, const void* fin, const void* gin, void* fout,
+                               void* gout, const DevStatus* st, int shape);
+TileLaunch launch_tile_f32, launch_tile_f16, launch_tile_bf16;
+TileLaunch launch_tile_cascaded_f32, launch_tile_cascaded_f16, launch_tile_cascaded_bf16;
+TileLaunch launch_tile_central_f32, launch_tile_central_f16, launch_tile_central_bf16;
 cudaError_t launch_fields(const Launch& L, const void* fin, const void* gin, const FieldPtrs& out);
 cudaError_t launch_pops(const Launch& L, const void* fin, const void* gin, float* f, float* g);
 cudaError_t launch_init(const Launch& L, const InitPtrs& in, void* fout, void* gout);

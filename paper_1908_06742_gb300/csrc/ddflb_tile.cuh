@@ -17,12 +17,14 @@ namespace ddflb {
 // A small lattice is bound by the launch and by the latency of one node's
 // update (about 0.5 us), not by any rate: one step per launch takes 2.0 us at
 // 64^2 FP32, four per launch 0.90 us a step, the redundant nodes included
-// (128^2 cavity 2.2 -> 1.25, 256^2 cavity 3.1 -> 2.2, periodic FP16 3.0 -> 1.7).
+// (128^2 cavity 2.2 -> 1.16, 256^2 cavity 3.2 -> 2.1, periodic BF16 2.5 -> 1.6;
+// cascaded 64^2 2.1 -> 1.12, central moments 2.0 -> 0.87, cascaded with a force
+// 256^2 cavity 3.5 -> 2.9).
 // Three or six steps per launch measured 0.99 and 1.03 at 64^2, eight 1.25.
 // Tile sizes are compile-time constants, so that the planes' offsets are
 // immediates and the divisions multiplications: with sizes as arguments 64^2
 // took 1.09 and the 256^2 cavity 2.6.
-template <typename S, int BC, bool FORCE, int TX, int TY, int T, int NTH>
+template <typename S, int BC, bool FORCE, int SM, int TX, int TY, int T, int NTH>
 __global__ void __launch_bounds__(NTH) k_tile(LbParams P, const S* __restrict__ fin,
                                                        const S* __restrict__ gin,
                                                        S* __restrict__ fout, S* __restrict__ gout,
@@ -91,7 +93,7 @@ __global__ void __launch_bounds__(NTH) k_tile(LbParams P, const S* __restrict__ 
           }
         }
       }
-      collide<FORCE, 0, sizeof(S) == 4>(P, x, y, df, dg);
+      collide<FORCE, SM, sizeof(S) == 4>(P, x, y, df, dg);
       if (l < T) {
 #pragma unroll
         for (int a = 0; a < 9; ++a) {
@@ -113,11 +115,11 @@ __global__ void __launch_bounds__(NTH) k_tile(LbParams P, const S* __restrict__ 
 
 namespace tile {
 
-template <typename S, int BC, bool FORCE, int TX, int TY, int NTH>
+template <typename S, int BC, bool FORCE, int SM, int TX, int TY, int NTH>
 cudaError_t go(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                const DevStatus* st) {
   constexpr int T = kTileSteps;
-  auto* kernel = k_tile<S, BC, FORCE, TX, TY, T, NTH>;
+  auto* kernel = k_tile<S, BC, FORCE, SM, TX, TY, T, NTH>;
   // two buffers of the tile with T - 1 nodes around it
   const int smem = 2 * 18 * (TX + 2 * T - 2) * (TY + 2 * T - 2) * (int)sizeof(S);
   static const cudaError_t attr =
@@ -137,32 +139,32 @@ cudaError_t go(const Launch& L, const void* fin, const void* gin, void* fout, vo
                             st);
 }
 
-template <typename S, int BC, bool FORCE>
+template <typename S, int BC, bool FORCE, int SM>
 cudaError_t go_shape(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                      const DevStatus* st, int shape) {
   switch (shape) {
-    case 0: return go<S, BC, FORCE, 8, 4, 160>(L, fin, gin, fout, gout, st);
-    case 1: return go<S, BC, FORCE, 8, 8, 256>(L, fin, gin, fout, gout, st);
-    case 2: return go<S, BC, FORCE, 16, 8, 320>(L, fin, gin, fout, gout, st);
-    case 3: return go<S, BC, FORCE, 16, 16, 512>(L, fin, gin, fout, gout, st);
-    default: return go<S, BC, FORCE, 32, 14, 768>(L, fin, gin, fout, gout, st);
+    case 0: return go<S, BC, FORCE, SM, 8, 4, 160>(L, fin, gin, fout, gout, st);
+    case 1: return go<S, BC, FORCE, SM, 8, 8, 256>(L, fin, gin, fout, gout, st);
+    case 2: return go<S, BC, FORCE, SM, 16, 8, 320>(L, fin, gin, fout, gout, st);
+    case 3: return go<S, BC, FORCE, SM, 16, 16, 512>(L, fin, gin, fout, gout, st);
+    default: return go<S, BC, FORCE, SM, 32, 14, 768>(L, fin, gin, fout, gout, st);
   }
 }
 
-template <typename S, int BC>
+template <typename S, int BC, int SM>
 cudaError_t go_force(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                      const DevStatus* st, int shape) {
-  return L.force ? go_shape<S, BC, true>(L, fin, gin, fout, gout, st, shape)
-                 : go_shape<S, BC, false>(L, fin, gin, fout, gout, st, shape);
+  return L.force ? go_shape<S, BC, true, SM>(L, fin, gin, fout, gout, st, shape)
+                 : go_shape<S, BC, false, SM>(L, fin, gin, fout, gout, st, shape);
 }
 
-template <typename S>
+template <typename S, int SM>
 cudaError_t go_bc(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                   const DevStatus* st, int shape) {
   switch (L.P_bc) {
-    case BC_PERIODIC: return go_force<S, BC_PERIODIC>(L, fin, gin, fout, gout, st, shape);
-    case BC_CAVITY: return go_force<S, BC_CAVITY>(L, fin, gin, fout, gout, st, shape);
-    default: return go_force<S, BC_CHANNEL>(L, fin, gin, fout, gout, st, shape);
+    case BC_PERIODIC: return go_force<S, BC_PERIODIC, SM>(L, fin, gin, fout, gout, st, shape);
+    case BC_CAVITY: return go_force<S, BC_CAVITY, SM>(L, fin, gin, fout, gout, st, shape);
+    default: return go_force<S, BC_CHANNEL, SM>(L, fin, gin, fout, gout, st, shape);
   }
 }
 

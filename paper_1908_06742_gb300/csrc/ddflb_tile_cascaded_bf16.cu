@@ -1,0 +1,9 @@
+// k_tile with the cascaded scalar model for __nv_bfloat16 storage (one translation unit per storage type).
+#include "ddflb_tile.cuh"
+
+namespace ddflb {
+cudaError_t launch_tile_cascaded_bf16(const Launch& L, const void* fin, const void* gin, void* fout,
+                                      void* gout, const DevStatus* st, int shape) {
+  return tile::go_bc<__nv_bfloat16, 2>(L, fin, gin, fout, gout, st, shape);
+}
+}  // namespace ddflb

@@ -4,6 +4,6 @@
 namespace ddflb {
 cudaError_t launch_tile_f16(const Launch& L, const void* fin, const void* gin, void* fout,
                           void* gout, const DevStatus* st, int shape) {
-  return tile::go_bc<__half>(L, fin, gin, fout, gout, st, shape);
+  return tile::go_bc<__half, 0>(L, fin, gin, fout, gout, st, shape);
 }
 }  // namespace ddflb
