@@ -300,10 +300,10 @@ ddflb_status ddflb_set_block(ddflb_ctx* c, int32_t block_x, int32_t block_y);
  * nx a multiple of 4; nodes next to a wall one by one; otherwise falls back to
  * 2, then 1);
  * 0 (default) = by size: four steps per launch on small lattices (about 256^2
- * at most, no time-dependent force), two on large ones (unforced MRT or SRT
- * scalar, from 1.4 to 10 million nodes on), single steps with two nodes per
- * thread between them and where a call or a residual check leaves some (16-bit
- * periodic ones of a million nodes with four).  All give bit-identical
+ * at most, no time-dependent force), two on large ones (from 1.4 to 10 million
+ * nodes on, no force field; 16-bit storage: MRT or SRT, no force), single steps
+ * with two nodes per thread between them and where a call or a residual check
+ * leaves some (16-bit periodic ones of a million nodes with four).  All give bit-identical
  * results; which is faster depends on the shape, so the autotuner times them. */
 ddflb_status ddflb_set_path(ddflb_ctx* c, int32_t path);
 

@@ -282,19 +282,25 @@ cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void*
 // kernel: FP32 periodic 1100^2 26.7 / 25.4, 1200^2 28.6 / 29.1, 2048^2 68 / 84;
 // FP32 cavity 1200^2 31.5 / 29.5, 1400^2 39.3 / 39.9; 16-bit cavity 2048^2 58.5 /
 // 56.1, 4096^2 210 / 246; 16-bit periodic 2048^2 54.3 / 49.3 (four nodes per
-// thread), 4096^2 180 / 186.
+// thread), 4096^2 180 / 186.  FP32 with a uniform force 1450^2 44.8 / 44.8, 2048^2
+// 78 / 85; forced cascaded 2048^2 93 / 88, 4096^2 322 / 351, 8192 x 4096 605 / 703.
 int64_t march_min_nodes(const Launch& L) {
+  if (L.P.smodel >= 2) return 10000000;
+  if (L.force) return 3000000;
   if (L.storage == 0) return L.P_bc == BC_PERIODIC ? 1400000 : 2000000;
   return quad_step_eligible(L) && L.P_bc == BC_PERIODIC ? 10000000 : 6000000;
 }
 
 // Rows per warp of the two-step kernel (ddflb_march.cuh), or 0 where steps go
-// one per launch: the y-slab contexts, forced lattices and central-moment
-// scalar models (whose collisions have no packed form), an explicit path, and
+// one per launch: the y-slab contexts, a force that depends on place or time,
+// 16-bit storage with a force or a central-moment model, an explicit path, and
 // lattices too small.
 int choose_march_rows(const ddflb_ctx* c) {
   const LbParams& P = c->L.P;
-  if (c->path != 0 || P.y0 != 0 || P.y1 != P.ny || c->L.force || P.smodel >= 2) return 0;
+  if (c->path != 0 || P.y0 != 0 || P.y1 != P.ny) return 0;
+  if ((c->L.force || P.smodel >= 2) &&
+      (c->L.storage != 0 || P.ffield != nullptr || c->p.force_omega != 0.0))
+    return 0;
   if ((int64_t)P.nx * P.ny < march_min_nodes(c->L)) return 0;
   // strips x chunks in waves of 15 warps an SM, plus most of a chunk at the end
   // while the last ones finish (FP32 8192^2, rows 16 / 32 / 64 / 128: 878, 853,
@@ -319,9 +325,12 @@ cudaError_t run_two(const ddflb_ctx* c, int src) {
   const size_t gofs = c->lay.gofs;
   const char* fi = (const char*)c->pops[src];
   char* fo = (char*)c->pops[src ^ 1];
-  auto* launch = c->L.storage == 0   ? launch_march2_f32
-                 : c->L.storage == 1 ? launch_march2_f16
-                                     : launch_march2_bf16;
+  auto* launch = c->L.storage == 1    ? launch_march2_f16
+                 : c->L.storage == 2  ? launch_march2_bf16
+                 : c->L.P.smodel == 2 ? launch_march2_cascaded
+                 : c->L.P.smodel == 3 ? launch_march2_central
+                 : c->L.force         ? launch_march2_forced
+                                      : launch_march2_f32;
   return launch(c->L, fi, fi + gofs, fo, fo + gofs, c->status, c->march_rows);
 }
 

@@ -67,12 +67,11 @@ cudaError_t launch_step_duo_f16(const Launch& L, const void* fin, const void* gi
 cudaError_t launch_step_duo_bf16(const Launch& L, const void* fin, const void* gin, void* fout,
                                  void* gout, const DevStatus* st, bool down);
 // two time steps in one launch (ddflb_march.cuh); rows: lattice rows per CTA
-cudaError_t launch_march2_f32(const Launch& L, const void* fin, const void* gin, void* fout,
-                              void* gout, DevStatus* st, int rows);
-cudaError_t launch_march2_f16(const Launch& L, const void* fin, const void* gin, void* fout,
-                              void* gout, DevStatus* st, int rows);
-cudaError_t launch_march2_bf16(const Launch& L, const void* fin, const void* gin, void* fout,
-                               void* gout, DevStatus* st, int rows);
+typedef cudaError_t MarchLaunch(const Launch& L, const void* fin, const void* gin, void* fout,
+                                void* gout, DevStatus* st, int rows);
+MarchLaunch launch_march2_f32, launch_march2_f16, launch_march2_bf16;
+// FP32 with a uniform force, with a central-moment scalar model
+MarchLaunch launch_march2_forced, launch_march2_cascaded, launch_march2_central;
 // several time steps per launch on small lattices (ddflb_tile.cuh): the tile
 // shapes it is built for, smallest first
 constexpr int kTileSteps = 4, kTileShapes = 5;

@@ -1,6 +1,6 @@
 // Two fused time steps per pass over memory (k_march2), one warp per strip of
-// the lattice (unforced MRT and SRT collisions): see the kernel's comment.  Included by one translation unit per
-// storage type, so that they compile in parallel.
+// the lattice: see the kernel's comment.  Included by one translation unit per
+// storage type and model, so that they compile in parallel.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -78,8 +78,8 @@ __device__ __forceinline__ F2 from_right(F2 v) {
 }
 
 // warps per SM (the register budget: 128 at 16, 168 at 12)
-template <typename S, int BC>
-constexpr int kMarchWarps = sizeof(S) == 4 && BC != BC_PERIODIC ? 12 : 16;
+template <typename S, int BC, bool FORCE = false, int SM = 0>
+constexpr int kMarchWarps = (sizeof(S) == 4 && BC != BC_PERIODIC) || FORCE || SM ? 12 : 16;
 
 template <typename S>
 constexpr size_t march_smem(int bc) {
@@ -107,11 +107,14 @@ constexpr size_t march_smem(int bc) {
 // 3 warps per scheduler) 76; in shared memory (126 registers, 4 per scheduler)
 // 79, 311 instructions per node and step against 553.  FP16 16384^2: 108 against
 // 91 of k_step_quad (16 warps an SM; 12: 97, 20 with spills: 78).  The walled
-// FP32 forms keep 12 warps (4096^2 cavity: 67; at 16, with spills: 60).
+// FP32 forms keep 12 warps (4096^2 cavity: 67; at 16, with spills: 60), and so do
+// those with a force or a central-moment model (8192 x 4096 periodic, us per step,
+// two nodes per thread -> this: forced MRT 691 -> 501, cascaded 695 -> 557, forced
+// cascaded 703 -> 605, central moments 691 -> 524).
 //
 // `strip` and rows [y0, y1) name the strip and chunk; shared: march_smem() bytes;
 // bars: STAGES mbarriers; wall: 12 floats; *timeout is set if a copy fails to arrive.
-template <typename S, int BC>
+template <typename S, int BC, bool FORCE = false, int SM = 0>
 __device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& K,
                                             const S* __restrict__ fin, const S* __restrict__ gin,
                                             S* __restrict__ fout, S* __restrict__ gout, int strip,
@@ -119,6 +122,10 @@ __device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& 
                                             float* s_wall, int* timeout) {
   using Io = PairIo<S>;
   constexpr bool COMP = sizeof(S) == 4;
+  static_assert(COMP || !(FORCE || SM), "16-bit storage: unforced MRT only");
+  // the force is the same at every node and step
+  const F2 Fx = make_float2(P.fx * P.fmod, P.fx * P.fmod);
+  const F2 Fy = make_float2(P.fy * P.fmod, P.fy * P.fmod);
   constexpr int NST = Io::STAGES, SEG = Io::SEG, W = kMarchStrip;
   S* const stage0 = reinterpret_cast<S*>(shared);
   // stage 0, the values handed on, the other stages, D: the outer lanes' reads one
@@ -303,7 +310,7 @@ __device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& 
           }
         }
       }
-      collide_pair<COMP>(K, df, dg);
+      collide_pair<COMP, FORCE, SM>(K, df, dg, Fx, Fy);
       if (sg) {
         // every lane has read this stage: refill it
         __syncwarp();
@@ -394,7 +401,7 @@ __device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& 
     }
     __syncwarp();
     if (y >= y0) {
-      collide_pair<COMP>(K, nf, ng);
+      collide_pair<COMP, FORCE, SM>(K, nf, ng, Fx, Fy);
       if (xa >= xs && xa < xe) {
         // (where nx is odd the last pair's second value lands in the row's padding)
         const int64_t o = (int64_t)y * P.pitch + xa;
@@ -422,8 +429,8 @@ __device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& 
   }
 }
 
-template <typename S, int BC>
-__global__ void __launch_bounds__(32, kMarchWarps<S, BC>)
+template <typename S, int BC, bool FORCE, int SM>
+__global__ void __launch_bounds__(32, kMarchWarps<S, BC, FORCE, SM>)
     k_march2(LbParams P, PairConst K, const S* __restrict__ fin, const S* __restrict__ gin,
              S* __restrict__ fout, S* __restrict__ gout, DevStatus* __restrict__ status,
              int rows) {
@@ -432,28 +439,28 @@ __global__ void __launch_bounds__(32, kMarchWarps<S, BC>)
   __shared__ float s_wall[12];  // cavity: the side walls' links in row i
   if (status->diverged) return;
   const int y0 = blockIdx.y * rows;
-  march_strip<S, BC>(P, K, fin, gin, fout, gout, blockIdx.x, y0, min(y0 + rows, P.ny), march_shared,
-                     s_bar, s_wall, &status->timeout);
+  march_strip<S, BC, FORCE, SM>(P, K, fin, gin, fout, gout, blockIdx.x, y0, min(y0 + rows, P.ny),
+                                march_shared, s_bar, s_wall, &status->timeout);
 }
 
 namespace march {
 
-template <typename S, int BC>
+template <typename S, int BC, bool FORCE, int SM>
 cudaError_t go(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                DevStatus* st, int rows) {
   const dim3 g(march_strips(BC, L.P.nx), (L.P.ny + rows - 1) / rows);
-  k_march2<S, BC><<<g, 32, march_smem<S>(BC), L.stream>>>(
+  k_march2<S, BC, FORCE, SM><<<g, 32, march_smem<S>(BC), L.stream>>>(
       L.P, make_pair_const(L.P), (const S*)fin, (const S*)gin, (S*)fout, (S*)gout, st, rows);
   return cudaGetLastError();
 }
 
-template <typename S>
+template <typename S, bool FORCE, int SM>
 cudaError_t go_bc(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                   DevStatus* st, int rows) {
   switch (L.P_bc) {
-    case BC_PERIODIC: return go<S, BC_PERIODIC>(L, fin, gin, fout, gout, st, rows);
-    case BC_CAVITY: return go<S, BC_CAVITY>(L, fin, gin, fout, gout, st, rows);
-    default: return go<S, BC_CHANNEL>(L, fin, gin, fout, gout, st, rows);
+    case BC_PERIODIC: return go<S, BC_PERIODIC, FORCE, SM>(L, fin, gin, fout, gout, st, rows);
+    case BC_CAVITY: return go<S, BC_CAVITY, FORCE, SM>(L, fin, gin, fout, gout, st, rows);
+    default: return go<S, BC_CHANNEL, FORCE, SM>(L, fin, gin, fout, gout, st, rows);
   }
 }
 
