@@ -284,10 +284,10 @@ ddflb_status ddflb_reduce_noalloc(const ddflb_params* p, const void* dev_state,
  * 64x2, 32x4, 64x4, 32x8, 64x1) with each kernel variant (path 1: one node per
  * thread; path 2, 16-bit storage with even nx only: two adjacent nodes per
  * thread with aligned 4-byte pair accesses), and path 3 (four nodes per
- * thread, its own 128x1 block) once where it applies, and path 0 once where it
- * takes two steps per launch, over trial_steps with
- * CUDA events, and keeps the fastest.  Runs on zeroed populations, so it OVERWRITES the state and
- * resets the step counter: call it before ddflb_init.  Synchronises. */
+ * thread, its own 128x1 block) and path 0 (whichever kernel it takes) once, over
+ * trial_steps with CUDA events, and keeps the fastest.  Runs on zeroed
+ * populations, so it OVERWRITES the state and resets the step counter: call it
+ * before ddflb_init.  Synchronises. */
 ddflb_status ddflb_autotune(ddflb_ctx* c, int32_t trial_steps, int32_t* block_x,
                             int32_t* block_y, int32_t* path, double* ms_per_step);
 /* Set the step kernel's block shape directly (e.g. from a cached tuning):

@@ -941,20 +941,31 @@ ddflb_status ddflb_autotune(ddflb_ctx* c, int32_t trial_steps, int32_t* block_x,
       }
     }
   }
-  // the automatic path, where it takes two steps per launch (at the default block)
+  // the automatic path: two or four steps per launch, or single ones (at the
+  // default block)
   c->path = 0;
+  c->L.block = dim3(128, 1, 1);
   c->march_rows = choose_march_rows(c);
-  if (c->march_rows > 0 && e == cudaSuccess) {
-    const int pairs = (trial_steps + 1) / 2;
+  c->tile = choose_tile(c);
+  if (e == cudaSuccess) {
+    const int per = c->march_rows > 0 ? 2 : c->tile >= 0 ? kTileSteps : 1;
+    const int launches = (trial_steps + per - 1) / per;
     for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
       if (rep == 1) e = cudaEventRecord(e0, s);
-      for (int i = 0; i < pairs && e == cudaSuccess; ++i) e = run_two(c, i & 1);
+      for (int i = 0; i < launches && e == cudaSuccess; ++i) {
+        const int src = i & 1;
+        char* fo = (char*)c->pops[src ^ 1];
+        e = per == 2            ? run_two(c, src)
+            : per == kTileSteps ? run_tile(c, src)
+                                : run_step(c, c->pops[src], (const char*)c->pops[src] + gofs, fo,
+                                           fo + gofs);
+      }
     }
     if (e == cudaSuccess) e = cudaEventRecord(e1, s);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-    ms *= (float)trial_steps / (2 * pairs);
+    ms *= (float)trial_steps / (per * launches);
     if (e == cudaSuccess && ms < best) {
       best = ms;
       bestb = dim3(128, 1, 1);
