@@ -444,7 +444,7 @@ template <typename S, int BC>
 __global__ void __launch_bounds__(32, kMarchWarps<S, BC>)
     k_batch_march(BatchArgs A, const int4* __restrict__ items, const PairConst* __restrict__ consts,
                   int src) {
-  extern __shared__ __align__(128) unsigned char march_shared[];
+  extern __shared__ __align__(16) unsigned char march_shared[];
   __shared__ __align__(8) uint64_t s_bar[PairIo<S>::STAGES];
   __shared__ float s_wall[12];
   __shared__ BatchInst sI;

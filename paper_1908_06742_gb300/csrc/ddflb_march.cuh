@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(32, kMarchWarps<S, BC, FORCE, SM>)
     k_march2(LbParams P, PairConst K, const S* __restrict__ fin, const S* __restrict__ gin,
              S* __restrict__ fout, S* __restrict__ gout, DevStatus* __restrict__ status,
              int rows) {
-  extern __shared__ __align__(128) unsigned char march_shared[];
+  extern __shared__ __align__(16) unsigned char march_shared[];
   __shared__ __align__(8) uint64_t s_bar[PairIo<S>::STAGES];
   __shared__ float s_wall[12];  // cavity: the side walls' links in row i
   if (status->diverged) return;
