@@ -246,9 +246,9 @@ namespace {
 // Smallest lattice that steps two nodes per thread in packed arithmetic: below it
 // one node per thread has more warps to hide latency with.  us per step, one node
 // -> two: FP32 cascaded 256^2 3.08 -> 3.10, 300^2 3.95 -> 3.66; BF16 96^2 1.98 ->
-// 2.19, 160^2 2.50 -> 2.40.
+// 2.19, 160^2 2.50 -> 2.40; FP32 channel 348 x 261 3.64 -> 3.69, 350^2 4.13 -> 3.95.
 int64_t duo_min_nodes(const Launch& L) {
-  if (L.storage == 0) return 85000;
+  if (L.storage == 0) return L.P_bc == BC_PERIODIC ? 85000 : 110000;
   return L.force || L.P.smodel >= 2 ? 20000 : 0;
 }
 

@@ -40,7 +40,7 @@ struct DuoIo<float> {
 // descending order; taken every other step where the two buffers exceed L2, so that
 // a step begins with the rows the last one ended with.  us per step, one node per
 // thread -> this:
-//   MRT FP32              420^2 5.15 -> 4.21   701^2 10.2 -> 8.5   1024^2 24.4 -> 20.6
+//   MRT FP32              420^2 5.15 -> 4.21   701^2 10.2 -> 8.5   1024^2 24.4 -> 20.4
 //   MRT BF16              420^2 4.62 -> 3.42   701^2 9.2 -> 6.6
 //   forced cascaded FP32  701^2 13.3 -> 10.6   1024^2 29.8 -> 23.5   4096^2 425 -> 350
 //   forced cascaded BF16  701^2 11.9 -> 9.1    1024^2 22.2 -> 17.2   4096^2 338 -> 258
@@ -48,7 +48,7 @@ struct DuoIo<float> {
 // whose groups next to a wall go node by node: 1024^2 19.6 -> 13.2, 2048^2 64.9 ->
 // 56.1.  Five CTAs per SM throughout: with four, forced cascaded BF16 4096^2 272
 // (and MRT FP32 1024^2 24.2; six 25.0, evict-first stores 21.2 against 20.4).
-template <typename S, int BC, bool FORCE, int SM>
+template <typename S, int BC, bool FORCE, int SM, int BX>
 __global__ void __launch_bounds__(128, 5)
     k_step_duo(LbParams P, PairConst K, const S* __restrict__ fin, const S* __restrict__ gin,
                S* __restrict__ fout, S* __restrict__ gout, const DevStatus* __restrict__ status,
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(128, 5)
   // 16-bit populations stay in storage units where the collision allows it
   constexpr bool UNITS = !COMP && (FORCE || SM != 0);
   const int nx = P.nx, ny = P.ny;
-  const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  const int x0 = 2 * (blockIdx.x * (BX ? BX : blockDim.x) + threadIdx.x);
   const int y = down ? ny - 1 - (int)blockIdx.y : (int)blockIdx.y;
   if (x0 >= nx || status->diverged) return;
   F2 df[9], dg[9];
@@ -154,14 +154,16 @@ template <typename S, int BC, bool FORCE, int SM>
 cudaError_t go(const Launch& L, const void* fin, const void* gin, void* fout, void* gout,
                const DevStatus* st, bool down) {
   // blocks of 128 pairs of one row, or of 64 or 32 where that leaves fewer threads
-  // without a node (350^2: 6 blocks of 32 a row instead of 2 of 128)
+  // without a node (350^2: 6 blocks of 32 a row instead of 2 of 128); the widest as a
+  // constant (1024^2 20.9 us per step with the width read at run time, 20.4 so)
   const int pairs = (L.P.nx + 1) / 2;
   int bx = 128;
   for (int b : {64, 32})
     if ((pairs + b - 1) / b * b < (pairs + bx - 1) / bx * bx) bx = b;
   const dim3 g((pairs + bx - 1) / bx, L.P.ny);
-  k_step_duo<S, BC, FORCE, SM><<<g, bx, 0, L.stream>>>(
-      L.P, make_pair_const(L.P), (const S*)fin, (const S*)gin, (S*)fout, (S*)gout, st, down);
+  auto* kernel = bx == 128 ? k_step_duo<S, BC, FORCE, SM, 128> : k_step_duo<S, BC, FORCE, SM, 0>;
+  kernel<<<g, bx, 0, L.stream>>>(L.P, make_pair_const(L.P), (const S*)fin, (const S*)gin,
+                                 (S*)fout, (S*)gout, st, down);
   return cudaGetLastError();
 }
 template <typename S, int BC, bool FORCE>

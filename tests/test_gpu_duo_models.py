@@ -29,7 +29,7 @@ def _run(D, cfg, fields, field, path, steps):
 # odd and even widths, blocks of 32, 64 and 128 pairs and one pair more, few columns
 @pytest.mark.parametrize("storage", ["fp32", "fp16", "bf16"])
 @pytest.mark.parametrize("bc", ["periodic", "cavity", "channel"])
-@pytest.mark.parametrize("nx,ny", [(3, 30001), (64, 1400), (129, 700), (257, 350), (258, 400),
+@pytest.mark.parametrize("nx,ny", [(3, 40001), (64, 1800), (129, 900), (257, 450), (258, 440),
                                    (350, 350), (701, 613), (1100, 1200)])
 def test_models_match_single_nodes(bc, storage, nx, ny):
     import torch
