@@ -40,8 +40,8 @@ def parse():
     ap.add_argument("--lb-steps", type=int, default=200, help="fused time steps per benchmark step")
     ap.add_argument("--storage", default="fp32", choices=["fp32", "fp16", "bf16"])
     ap.add_argument("--step-path", type=int, default=0, choices=[0, 1, 2, 3],
-                    help="step kernel (ddflb_set_path): 0 default (groups of 4 nodes for "
-                         "16-bit storage), 1 one node per thread, 2 node pairs, 3 groups of 4")
+                    help="step kernel (ddflb_set_path): 0 default (by size: 4 or 2 steps per "
+                         "launch, or node pairs), 1 one node per thread, 2 node pairs, 3 groups of 4")
     ap.add_argument("--scalar-model", default="mrt", choices=["mrt", "srt", "cascaded", "central"],
                     help="scalar collision (Sec. 3 MRT, App. B SRT, App. C cascaded, App. D central)")
     ap.add_argument("--no-e2e", action="store_true")
@@ -252,18 +252,33 @@ def run_reference(args, world, rank):
 
 
 # ------------------------------------------------------------------ GPU arm
+def step_kernel(args):
+    """(name, time steps per launch) of the kernel that runs the Taylor-Green
+    context's steps for --step-path (unforced periodic n x n lattice; the rules of
+    run_step, choose_tile and march_min_nodes in csrc/ddflb_api.cu)."""
+    n, nodes, half = args.n, args.n * args.n, args.storage != "fp32"
+    plain = args.scalar_model in ("mrt", "srt")
+    if args.step_path == 0:
+        if -(-n // 32) * -(-n // 14) <= 152:
+            return "k_tile", 4
+        quad = half and plain and n % 4 == 0
+        two = (1.4e6 if not half else 1e7 if quad else 6e6) if plain else 1e7
+        if nodes >= two and (plain or not half):
+            return "k_march2", 2
+        if quad and nodes > 900000:
+            return "k_step_quad", 1
+        if nodes >= (85000 if not half else 0 if plain else 20000):
+            return "k_step_duo", 1
+        return "k_step", 1
+    if args.step_path == 3 and half and n % 4 == 0 and plain:
+        return "k_step_quad", 1
+    if args.step_path in (2, 3) and half and n % 2 == 0 and plain:
+        return "k_step_pair", 1
+    return "k_step", 1
+
+
 def step_kernel_name(args):
-    """The step kernel the Taylor-Green context runs for --step-path (the
-    paired kernel takes 16-bit storage, even n and the MRT / SRT scalar)."""
-    if (args.step_path in (0, 3) and args.storage != "fp32" and args.n % 4 == 0
-            and args.scalar_model in ("mrt", "srt")):
-        return "k_step_quad"
-    # the Taylor-Green lattice is periodic: there the default takes pairs when
-    # n is not a multiple of 4
-    pair = args.step_path in (2, 3) or (args.step_path == 0 and args.storage != "fp32")
-    if pair and args.storage != "fp32" and args.n % 2 == 0 and args.scalar_model in ("mrt", "srt"):
-        return "k_step_pair"
-    return "k_step"
+    return step_kernel(args)[0]
 
 
 def traffic_per_launch(args, n_cells):
@@ -368,11 +383,15 @@ def run_ours(args, world, rank, local):
         total_ms = sum(a.elapsed_time(c) for a, _, c in ev)
         step_ms = sum(a.elapsed_time(b) for a, b, _ in ev)
         total_ms = max_over_ranks(world, total_ms)
-        launches = args.steps * (lb + 1)
+        # lb steps take lb // T launches of T steps and single ones for the rest; then fields
+        T_launch = step_kernel(args)[1]
+        launches = args.steps * (lb // T_launch + lb % T_launch + 1)
 
         cells = n * n
         value = world * cells * lb * args.steps / (total_ms / 1e3) / 1e6
-        kernel_s = step_ms / 1e3 / (lb * args.steps)     # average k_step launch duration
+        # average duration of a launch, which reads and writes every population once
+        # (n steps per launch: the update rate is n times the roofline's bytes)
+        kernel_s = step_ms / 1e3 / ((lb // T_launch + lb % T_launch) * args.steps)
         algo_bytes = BYTES_PER_CELL[args.storage] * cells
         peak, kind = peaks()
         achieved = algo_bytes / kernel_s / 1e9
@@ -424,7 +443,7 @@ def run_ours(args, world, rank, local):
                    "hbm_pct": round(100 * achieved / peak, 1)},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "peak_kind": kind,
-                     "kernel": step_kernel_name(args),
+                     "kernel": step_kernel_name(args), "steps_per_launch": T_launch,
                      "algorithmic_bytes_per_launch": algo_bytes,
                      "traffic": traffic_per_launch(args, cells),
                      "traffic_source": traffic_source(step_kernel_name(args) + "_" + args.storage
@@ -439,6 +458,21 @@ def run_ours(args, world, rank, local):
         "checks": {"mass": stats["mass"], "diverged": stats["diverged"]},
     }
     print(json.dumps(line))
+
+
+def batch_launches(t0, lb, K=100):
+    """(launches, passes over the populations) of one chunk of lb steps from step t0
+    under schedule 1: two steps per launch between the checks (every K steps),
+    single ones around them, with the sums and the check kernel after a check
+    step, then the state-time update."""
+    n, passes, k = 1, 0, 0
+    while k < lb:
+        t = t0 + k
+        two = k + 1 < lb and t % K and (t + 1) % K
+        n += 1 if t % K else 2 if t == 0 else 3
+        passes += 1
+        k += 2 if two else 1
+    return n, passes
 
 
 def batch_configs(args, rank, world):
@@ -513,7 +547,12 @@ def run_batch(args, world, rank, local):
         value = job_cells * lb * args.steps / (total_ms / 1e3) / 1e6
         peak, kind = peaks()
         # this rank's kernel against this GPU's copy peak
-        achieved = 144 * cells * lb * args.steps / (local_ms / 1e3) / 1e9
+        # every pass reads and writes the populations once (schedule 1: mostly two
+        # steps per pass)
+        chunks = [batch_launches((args.warmup + k) * lb, lb) if tune["choice"][3] else (1, lb)
+                  for k in range(args.steps)]
+        passes = sum(c[1] for c in chunks)
+        achieved = 144 * cells * passes / (local_ms / 1e3) / 1e9
         # per-instance flags of the whole job, in global order, on rank 0
         flags = gather_indexed({i: int(f) for i, f in zip(mine, st["flags"])}, world)
         e2e = None
@@ -550,18 +589,17 @@ def run_batch(args, world, rank, local):
                    "l2": f"{288 * cells / 1e9:.1f} GB of populations on rank 0"},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "peak_kind": kind,
-                     "kernel": "k_batch" if tune["choice"][3] == 0 else "k_batch_tile",
-                     # bytes per node-step from a 64-cavity capture, times this launch's
-                     # node-steps (traffic grows in proportion: every node-step moves the
-                     # same 18 planes)
-                     "algorithmic_bytes_per_launch": 144 * cells * lb,
-                     "traffic": traffic_record("k_batch_fp32", cells * lb),
-                     "traffic_source": traffic_source("k_batch_fp32", "node-steps of this launch")},
+                     "kernel": "k_batch" if tune["choice"][3] == 0 else "k_batch_march",
+                     "algorithmic_bytes_per_chunk": 144 * cells * chunks[0][1],
+                     # bytes per node-step of schedule 0 from a 64-cavity capture, times a
+                     # chunk's node-steps (every node-step moves the same 18 planes)
+                     "traffic": traffic_record("k_batch_fp32", cells * lb)
+                     if tune["choice"][3] == 0 else None,
+                     "traffic_source": traffic_source("k_batch_fp32", "node-steps of a chunk")
+                     if tune["choice"][3] == 0 else None},
         "cpu_baseline": None, "e2e": e2e,
-        # schedule 0: one cooperative launch per chunk of lb steps; schedule 1: per
-        # step the node kernel, the sums kernel and the check kernel, then the
-        # state-time update
-        "gpu_launches": args.steps * (1 if tune["choice"][3] == 0 else 3 * lb + 1),
+        # schedule 0: one cooperative launch per chunk of lb steps
+        "gpu_launches": sum(c[0] for c in chunks),
         "clocks": clk,
         "checks": {"flags_nonzero": int(sum(f != 0 for f in flags)), "instances": len(flags),
                    "status": int(st["status"])},
@@ -843,8 +881,10 @@ def run_sweep(args, world, rank, local):
                 del lat
             torch.cuda.empty_cache()
             bpc = BYTES_PER_CELL[st]
-            gbs = bpc * n * n * lb / (ms / 1e3) / 1e9
-            rows.append({"n": n, "storage": st, "kernel": step_kernel_name(a),
+            kernel, steps_per_launch = step_kernel(a)
+            gbs = bpc * n * n * lb / steps_per_launch / (ms / 1e3) / 1e9
+            rows.append({"n": n, "storage": st, "kernel": kernel,
+                         "steps_per_launch": steps_per_launch,
                          "mlups": round(world * n * n * lb / (ms / 1e3) / 1e6, 1),
                          "gbs": round(gbs, 1), "frac": round(gbs / peak, 4),
                          "l2_resident": bpc * n * n < 129e6, "diverged": bool(diverged)})

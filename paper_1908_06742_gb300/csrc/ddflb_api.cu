@@ -194,9 +194,8 @@ struct ddflb_ctx {
   float* stage;
   int64_t step;
   int64_t snap_step;  // step at which uprev was last written (-1: none)
-  int path;           // step kernel: 0 default (large lattices: two steps per launch; 16-bit storage: groups of 4 nodes, else
-                      // pairs on a periodic lattice, where eligible; else one node),
-                      // 1 one node per thread, 2 paired nodes, 3 groups of 4 nodes
+  int path;           // step kernel: 0 by the lattice's size (run_step, choose_tile,
+                      // choose_march_rows); 1 one node per thread, 2 pairs, 3 groups of 4
   float* stage_out;   // output staging area (host I/O)
   cudaStream_t io_up, io_down;  // streams of host uploads / downloads (null: the context stream)
   cudaEvent_t ev_in_free, ev_in_ready, ev_out_ready, ev_out_free;  // host-I/O ordering
