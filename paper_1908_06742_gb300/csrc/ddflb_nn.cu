@@ -1886,8 +1886,11 @@ ddflb_status ddflb_nn_conv3x3_wgrad(const void* X, int32_t B, int32_t H, int32_t
   a.units = (int)(per * B);
   // the GEMM's slices: ceil(P / splits) pixels, rounded up to 64
   const int64_t kchunk = ((P + splits - 1) / splits + 63) / 64 * 64;
-  const int slices = (int)((P + kchunk - 1) / kchunk);
+  int slices = (int)((P + kchunk - 1) / kchunk);
   a.per_slice = a.segment ? (int)(kchunk / U) : (a.units + slices - 1) / slices;
+  // (padded rows: their units may fill fewer slices of that many; a slice without
+  // a unit would leave its accumulators as tensor memory was)
+  slices = (a.units + a.per_slice - 1) / a.per_slice;
   a.ntn = Ci == 16 ? 1 : Ci / 32;
   a.partial = partial;
   const int chx = Ci == 16 ? 2 : 4;
