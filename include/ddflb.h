@@ -546,6 +546,12 @@ ddflb_status ddflb_nn_conv3x3_dgrad(const void* G, int32_t B, int32_t H, int32_t
 ddflb_status ddflb_nn_conv3x3_wgrad(const void* X, int32_t B, int32_t H, int32_t W, int32_t Ci,
                                     int32_t csx, const void* G, int32_t Co, int32_t csg, float* dW,
                                     int32_t splits, float* partial, void* stream);
+/* Whether the three calls above take a layer (1) or refuse its channels or its
+ * image with EINVAL (0), so that a caller can fall back on im2col + GEMM: form 0
+ * conv3x3_narrow (C inputs, N outputs), 1 conv3x3_dgrad (C = Co, N = Ci), 2
+ * conv3x3_wgrad (C = Ci, N = Co).  Rows that are no multiple of 128 (form 2: of
+ * 64) need (H + 8) (W + 2)^2 < 2^32. */
+int32_t ddflb_nn_conv3x3_takes(int32_t form, int32_t B, int32_t H, int32_t W, int32_t C, int32_t N);
 /* Weights of the adjoint convolution: Wf[ci][t][co] = Wt[co][8 - t][ci]
  * (BF16, Wt [Co][9][Ci] -> Wf [Ci][9][Co]), so that dX = conv3x3(dY, Wf)
  * with C = Co and N = Ci is the input gradient of Y = conv3x3(X, Wt). */

@@ -1607,6 +1607,31 @@ bool narrow_args(narrow::Args* a, const void* X, int B, int H, int W, int C, int
   return false;
 }
 
+// The channels' rule of the narrow kernels and whether a tile of the image fits
+// (bn: outputs per tile, 32 for the input gradient).
+bool narrow_fits(int B, int H, int W, int C, int N, int bn) {
+  if ((C != 16 && C != 32 && C != 64) || (int64_t)B * H * W > INT32_MAX) return false;
+  narrow::Args a;
+  GemmArgs g{};
+  g.N = N;
+  return narrow_args(&a, nullptr, B, H, W, C, C, nullptr, bn, 1, g);
+}
+
+// The channels that the weight gradient takes, and the images: positions are
+// divided by the padded rows' length with one 32-bit multiplication.
+bool wgrad_channels(int Ci, int Co) {
+  return Ci > 0 && (Ci == 16 || Ci % 32 == 0) && Co > 0 && Co % 8 == 0 && Co <= 128;
+}
+
+bool wgrad_image(int B, int H, int W) {
+  constexpr int U = wgrad::UNIT;
+  const bool segment = W % U == 0;
+  const int64_t pitch = W + 2, P = (int64_t)B * H * W;
+  const int64_t per = segment ? (int64_t)H * (W / U) : (H * pitch + U - 1) / U;
+  return P <= INT32_MAX && per * B <= INT32_MAX / 512 &&
+         (segment || ((int64_t)H + 8) * pitch * pitch < (int64_t)1 << 32);
+}
+
 template <int CH, int BN, bool SEP, int MT>
 ddflb_status narrow_run(const narrow::Args& a, cudaStream_t s) {
   auto* kernel = narrow::k_conv_narrow<CH, BN, SEP, MT>;
@@ -1860,8 +1885,8 @@ ddflb_status ddflb_nn_conv3x3_wgrad(const void* X, int32_t B, int32_t H, int32_t
                                     int32_t splits, float* partial, void* stream) {
   if (!X || !G || !dW || !partial || B <= 0 || H <= 0 || W <= 0 || splits < 1)
     return bad("conv3x3_wgrad: bad arguments");
-  if ((Ci != 16 && Ci % 32) || Ci <= 0 || Co % 8 || Co <= 0 || Co > 128 || csx < Ci || csg < Co ||
-      csx % 8 || csg % 8 || ((uintptr_t)X % 16) || ((uintptr_t)G % 16) || ((uintptr_t)partial % 16))
+  if (!wgrad_channels(Ci, Co) || csx < Ci || csg < Co || csx % 8 || csg % 8 ||
+      ((uintptr_t)X % 16) || ((uintptr_t)G % 16) || ((uintptr_t)partial % 16))
     return bad("conv3x3_wgrad: Ci must be 16 or a multiple of 32, Co a multiple of 8 up to 128, "
                "the strides multiples of 8, X, G and partial 16-byte aligned");
   wgrad::Args a{};
@@ -1879,9 +1904,7 @@ ddflb_status ddflb_nn_conv3x3_wgrad(const void* X, int32_t B, int32_t H, int32_t
   a.inv_pitch = 0xffffffffu / (uint32_t)a.pitch + 1u;
   const int64_t P = (int64_t)B * H * W;
   const int64_t per = a.segment ? (int64_t)H * (W / U) : ((int64_t)H * a.pitch + U - 1) / U;
-  if (P > INT32_MAX || per * B > INT32_MAX / 512 ||
-      (!a.segment && ((int64_t)H + 8) * a.pitch * a.pitch >= (int64_t)1 << 32))
-    return bad("conv3x3_wgrad: image too large");
+  if (!wgrad_image(B, H, W)) return bad("conv3x3_wgrad: image too large");
   a.per_img = (int)per;
   a.units = (int)(per * B);
   // the GEMM's slices: ceil(P / splits) pixels, rounded up to 64
@@ -1916,6 +1939,13 @@ ddflb_status ddflb_nn_conv3x3_wgrad(const void* X, int32_t B, int32_t H, int32_t
   k_splitk_reduce<<<grid_for((int64_t)Co * 9 * Ci), 256, 0, s>>>(partial, slices, Co, 9 * Ci, dW,
                                                                  9 * Ci, nullptr, 0, 0);
   return launched("conv3x3_wgrad sum");
+}
+
+int32_t ddflb_nn_conv3x3_takes(int32_t form, int32_t B, int32_t H, int32_t W, int32_t C,
+                               int32_t N) {
+  if (form < 0 || form > 2 || B <= 0 || H <= 0 || W <= 0 || N <= 0) return 0;
+  if (form == 2) return wgrad_channels(C, N) && wgrad_image(B, H, W);
+  return narrow_fits(B, H, W, C, N, form == 1 || N <= 32 ? 32 : 64);
 }
 
 ddflb_status ddflb_nn_set_conv_path(int32_t path) {

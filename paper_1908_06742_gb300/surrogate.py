@@ -130,6 +130,12 @@ class UNet:
             ("d1a", 0, V(A, "cat1"), V(A, "d1a"), V(G, "cat1"), V(G, "d1a")),
             ("d1b", 0, V(A, "d1a"), V(A, "d1b"), V(G, "d1a"), V(G, "d1b")),
         ]
+        # the layers that the library's kernels take straight from the activation
+        # (forward, input gradient, weight gradient); the others: im2col + GEMM
+        takes = lambda form, lv, C, N: bool(
+            self.lib.ddflb_nn_conv3x3_takes(form, B, *L[lv], C, N))
+        self.direct = {n: (takes(0, lv, vi.C, vo.C), takes(1, lv, vo.C, vi.C),
+                           takes(2, lv, vi.C, vo.C)) for n, lv, vi, vo, _, _ in self.layers}
         P0 = B * H * W
         kmax = max(9 * ci for n, ci, co in self.specs if n != "head")
         ci_of = {n: ci for n, ci, _ in self.specs}
@@ -170,15 +176,6 @@ class UNet:
         return (128 % bw == 0 and (W < 128 or W % 128 == 0) and H % bh == 0
                 and bw * bh * bb == 128 and self.B % bb == 0)
 
-    def _narrow_ok(self, C, W, bn):
-        """ddflb_nn_conv3x3_narrow / _dgrad take this layer: 16, 32 or 64 input
-        channels, two tiles (with halo) and the weights of bn outputs in shared
-        memory."""
-        if not self.implicit or C not in (16, 32, 64):
-            return False
-        npos = 390 if W % 128 == 0 else 128 + 2 * (W + 2) + 2
-        return 2 * C * (9 * bn + 2 * npos) <= 226 * 1024
-
     def _conv_fwd(self, name, lv, vin, vout):
         p = self.p[name]
         H, W = self.L[lv]
@@ -190,7 +187,7 @@ class UNet:
                                           co, None, 0, vout.ptr, vout.cs, p["b"].data_ptr(),
                                           LEAKY, 0, self.s))
             return
-        if self._narrow_ok(ci, W, 32 if co <= 32 else 64):
+        if self.implicit and self.direct[name][0]:
             _ck(self.lib.ddflb_nn_conv3x3_narrow(vin.ptr, self.B, H, W, ci, vin.cs,
                                                  p["wb"].data_ptr(), co, None, 0, vout.ptr,
                                                  vout.cs, p["b"].data_ptr(), LEAKY, 0, self.s))
@@ -209,7 +206,7 @@ class UNet:
         _ck(self.lib.ddflb_nn_act_bwd(gout.ptr, vout.ptr, P, co, gout.cs, vout.cs, LEAKY, gbf, co,
                                       self.s))
         _ck(self.lib.ddflb_nn_bias_grad(gout.ptr, P, co, gout.cs, p["gb"].data_ptr(), self.s))
-        if self.implicit and (ci == 16 or ci % 32 == 0) and co % 8 == 0 and co <= 128:
+        if self.implicit and self.direct[name][2]:
             # dW [co][9ci] from the activation and the gradient as they are
             _ck(self.lib.ddflb_nn_conv3x3_wgrad(vin.ptr, self.B, H, W, ci, vin.cs, gbf, co, co,
                                                 p["gw"].data_ptr(),
@@ -231,7 +228,7 @@ class UNet:
             _ck(self.lib.ddflb_nn_conv3x3(gbf, self.B, H, W, co, co, p["wT"].data_ptr(), ci,
                                           gin.ptr, gin.cs, None, 0, None, 0, 0, self.s))
             return
-        if self._narrow_ok(co, W, 32):
+        if self.implicit and self.direct[name][1]:
             # dX tap by tap, without the patch columns of the gradient
             _ck(self.lib.ddflb_nn_conv3x3_dgrad(gbf, self.B, H, W, co, co, p["wb"].data_ptr(), ci,
                                                 gin.ptr, gin.cs, self.s))
