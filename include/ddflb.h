@@ -291,7 +291,10 @@ ddflb_status ddflb_reduce_noalloc(const ddflb_params* p, const void* dev_state,
 ddflb_status ddflb_autotune(ddflb_ctx* c, int32_t trial_steps, int32_t* block_x,
                             int32_t* block_y, int32_t* path, double* ms_per_step);
 /* Set the step kernel's block shape directly (e.g. from a cached tuning):
- * block_x a multiple of 32, 32..256 threads in all. */
+ * block_x a multiple of 32, 32..256 threads in all.  It holds for the init and
+ * output kernels and for the steps of paths 1 and 2; path 0 takes it where it
+ * steps one node per thread, its other kernels have shapes of their own.  A
+ * lattice of more than 65535 rows needs block_y > 1. */
 ddflb_status ddflb_set_block(ddflb_ctx* c, int32_t block_x, int32_t block_y);
 /* Step kernel variant: 1 one node per thread; 2 paired nodes, two adjacent
  * nodes per thread with aligned 4-byte pair accesses (16-bit storage, even nx,

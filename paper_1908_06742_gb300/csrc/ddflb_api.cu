@@ -256,11 +256,16 @@ cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void*
   const int64_t nodes = (int64_t)c->L.P.nx * c->L.P.ny;
   // steps alternate their direction where the two buffers do not fit L2 together
   const bool down = 2 * c->lay.pops_bytes > (size_t)80 << 20 && fin == c->pops[1];
-  const bool quad = quad_step_eligible(c->L);
+  // the kernels with one block row per lattice row end at the largest grid; beyond it
+  // blocks of several rows (ddflb_set_block) step the lattice.  (A row offset in
+  // k_step_duo instead cost its other lattices up to 1 %: 1023 x 767 FP16 1940 ->
+  // 1959 us per 200 steps.)
+  const bool tall = c->path == 0 && c->L.P.ny > kMaxGridY;
+  const bool quad = quad_step_eligible(c->L) && !tall;
   // two nodes per thread in packed arithmetic (unforced MRT 16-bit periodic lattices:
   // until the four-node kernel's wider accesses pay; 1024^2 11.65 us per step
   // against 12.0, 700^2 7.65 against 6.8)
-  if (c->path == 0 && whole && nodes >= duo_min_nodes(c->L) &&
+  if (c->path == 0 && whole && !tall && nodes >= duo_min_nodes(c->L) &&
       !(quad && c->L.P_bc == BC_PERIODIC && nodes > 900000)) {
     auto* launch = c->L.storage == 0   ? launch_step_duo_f32
                    : c->L.storage == 1 ? launch_step_duo_f16
@@ -270,7 +275,9 @@ cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void*
   // 16-bit storage steps node groups by default (wider accesses; bit-identical)
   if ((c->path == 3 || c->path == 0) && quad)
     return launch_step_quad(c->L, fin, gin, fout, gout, c->status, c->path == 0 && down);
-  const bool pair = c->path == 2 || c->path == 3;
+  // (with walls the paired kernel is no faster than one node per thread)
+  const bool pair = c->path == 2 || c->path == 3 ||
+                    (tall && c->L.storage != 0 && c->L.P_bc == BC_PERIODIC);
   if (pair && pair_step_eligible(c->L))
     return launch_step_pair(c->L, fin, gin, fout, gout, c->status);
   return launch_step(c->L, fin, gin, fout, gout, c->status);

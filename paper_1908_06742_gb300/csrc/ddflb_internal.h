@@ -14,6 +14,7 @@ inline int march_strips(int bc, int nx) {
   if (bc == BC_CAVITY) return nx <= 64 ? 1 : 1 + (nx - 64 + kMarchStrip - 1) / kMarchStrip;
   return (nx + kMarchStrip - 1) / kMarchStrip;
 }
+constexpr int kMaxGridY = 65535;  // blocks of a grid in y
 constexpr int kReduceThreads = 256;
 constexpr int kReduceBlocks = 608;  // 4 per SM on a 152-SM GB300; fixed for deterministic sums
 
