@@ -19,6 +19,7 @@
 
 #include "../../include/ddflb.h"
 #include "ddflb_internal.h"
+#include "ddflb_smem.h"
 
 namespace ddflb {
 namespace nn {
@@ -1495,13 +1496,9 @@ int sm_count() {
 
 template <int BN>
 ddflb_status gemm_tcp_bn(const GemmArgs& g, int tm, int tn, int tz, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_gemm_tcp<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tcp::Cfg<BN>::SMEM) != cudaSuccess)
-      return launched("gemm tcgen05 attribute");
-    attr = true;
-  }
+  static ddflb::SharedLimit limit;
+  if (limit.raise((const void*)k_gemm_tcp<BN>, tcp::Cfg<BN>::SMEM) != cudaSuccess)
+    return launched("gemm tcgen05 attribute");
   CUtensorMap ma, mb;
   if (!make_map(&ma, g.A, g.M, g.K, g.lda, tc::BM) || !make_map(&mb, g.B, g.N, g.K, g.ldb, BN))
     return bad("gemm: TMA tensor map encoding failed");
@@ -1541,13 +1538,9 @@ ddflb_status conv_tcp_bn(GemmArgs g, const void* X, int B, int cs, cudaStream_t 
   // reads cost more than the loads they save, and the per-tap boxes are faster
   if (g_conv_path == 0 && cpt >= 2 && g.conv_bw == 128 && g.conv_bh == 1 && g.conv_bb == 1 &&
       ag >= 2) {
-    static bool battr = false;
-    if (!battr) {
-      if (cudaFuncSetAttribute(k_gemm_tcp<BN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               tcp::SMEM_MAX) != cudaSuccess)
-        return launched("conv tcgen05 band attribute");
-      battr = true;
-    }
+    static ddflb::SharedLimit blimit;
+    if (blimit.raise((const void*)k_gemm_tcp<BN, true>, tcp::SMEM_MAX) != cudaSuccess)
+      return launched("conv tcgen05 band attribute");
     CUtensorMap ma, mb;
     g.conv_ag = ag;
     g.conv_bs = bs;
@@ -1559,13 +1552,9 @@ ddflb_status conv_tcp_bn(GemmArgs g, const void* X, int B, int cs, cudaStream_t 
     }
     // a band map the driver does not encode: per-tap boxes below
   }
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_gemm_tcp<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tcp::Cfg<BN>::SMEM) != cudaSuccess)
-      return launched("conv tcgen05 attribute");
-    attr = true;
-  }
+  static ddflb::SharedLimit limit;
+  if (limit.raise((const void*)k_gemm_tcp<BN>, tcp::Cfg<BN>::SMEM) != cudaSuccess)
+    return launched("conv tcgen05 attribute");
   g.conv_ag = 0;
   g.conv_bs = 0;
   CUtensorMap ma, mb;
@@ -1635,9 +1624,9 @@ bool wgrad_image(int B, int H, int W) {
 template <int CH, int BN, bool SEP, int MT>
 ddflb_status narrow_run(const narrow::Args& a, cudaStream_t s) {
   auto* kernel = narrow::k_conv_narrow<CH, BN, SEP, MT>;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tcp::SMEM_MAX);
-  if (attr != cudaSuccess) return bad("narrow convolution: shared memory attribute");
+  static ddflb::SharedLimit limit;
+  if (limit.raise((const void*)kernel, tcp::SMEM_MAX) != cudaSuccess)
+    return launched("narrow convolution attribute");
   const int smem = 9 * CH * BN * 16 + a.nbuf * CH * a.npos * 16;
   const int per = sm_count() / a.ntn;
   kernel<<<(a.tiles < per ? a.tiles : per) * a.ntn, narrow::THREADS, smem, s>>>(a);
@@ -1669,13 +1658,9 @@ ddflb_status narrow_fwd(const void* X, int B, int H, int W, int cs, const void* 
 
 template <int BN>
 ddflb_status gemm_tc_bn(const GemmArgs& g, dim3 grid, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_gemm_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::Cfg<BN>::SMEM) != cudaSuccess)
-      return launched("gemm tcgen05 attribute");
-    attr = true;
-  }
+  static ddflb::SharedLimit limit;
+  if (limit.raise((const void*)k_gemm_tc<BN>, tc::Cfg<BN>::SMEM) != cudaSuccess)
+    return launched("gemm tcgen05 attribute");
   CUtensorMap ma, mb;
   if (!make_map(&ma, g.A, g.M, g.K, g.lda, tc::BM) || !make_map(&mb, g.B, g.N, g.K, g.ldb, BN))
     return bad("gemm: TMA tensor map encoding failed");
@@ -1926,13 +1911,9 @@ ddflb_status ddflb_nn_conv3x3_wgrad(const void* X, int32_t B, int32_t H, int32_t
   while (a.nbuf > 2 && a.nbuf * buf + slack > tcp::SMEM_MAX / 2) --a.nbuf;  // two CTAs per SM
   cudaStream_t s = (cudaStream_t)stream;
   auto* kernel = chx == 2 ? wgrad::k_conv_wgrad<2> : wgrad::k_conv_wgrad<4>;
-  static const cudaError_t attr[2] = {
-      cudaFuncSetAttribute(wgrad::k_conv_wgrad<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           tcp::SMEM_MAX / 2),
-      cudaFuncSetAttribute(wgrad::k_conv_wgrad<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           tcp::SMEM_MAX / 2)};
-  if (attr[0] != cudaSuccess || attr[1] != cudaSuccess)
-    return bad("conv3x3_wgrad: shared memory attribute");
+  static ddflb::SharedLimit limit[2];
+  if (limit[chx == 4].raise((const void*)kernel, tcp::SMEM_MAX / 2) != cudaSuccess)
+    return launched("conv3x3_wgrad attribute");
   kernel<<<slices * a.ntn * 3, wgrad::THREADS, a.nbuf * buf + slack, s>>>(a);
   ddflb_status st = launched("conv3x3_wgrad");
   if (st != DDFLB_OK) return st;

@@ -6,6 +6,7 @@
 
 #include "ddflb_device.cuh"
 #include "ddflb_internal.h"
+#include "ddflb_smem.h"
 
 namespace ddflb {
 
@@ -122,9 +123,9 @@ cudaError_t go(const Launch& L, const void* fin, const void* gin, void* fout, vo
   auto* kernel = k_tile<S, BC, FORCE, SM, TX, TY, T, NTH>;
   // two buffers of the tile with T - 1 nodes around it
   const int smem = 2 * 18 * (TX + 2 * T - 2) * (TY + 2 * T - 2) * (int)sizeof(S);
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (attr != cudaSuccess) return attr;
+  static SharedLimit limit;
+  const cudaError_t e = limit.raise((const void*)kernel, smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((L.P.nx + TX - 1) / TX, (L.P.ny + TY - 1) / TY);
   cfg.blockDim = dim3(NTH);
