@@ -310,12 +310,22 @@ int choose_march_rows(const ddflb_ctx* c) {
   if ((int64_t)P.nx * P.ny < march_min_nodes(c->L)) return 0;
   // strips x chunks in waves of 15 warps an SM, plus most of a chunk at the end
   // while the last ones finish (FP32 8192^2, rows 16 / 32 / 64 / 128: 878, 853,
-  // 870, 1023 us per step; 4096^2: 231, 237, 261, 325)
+  // 870, 1023 us per step; 4096^2: 231, 237, 261, 325).  The periodic FP32 form,
+  // whose 15 warps an SM are the most, takes 32 rows at most: with more, strips
+  // drift apart and read their neighbours' columns from memory again, by how much
+  // differs from one GPU to another (thousand million node updates a second at 32 /
+  // 48 / 64 rows: 16384^2 81.4 / 81.8 / 80.0 on one, 81.4 / 81.4 / 72.0 on another,
+  // 12288^2 81.0 / 80.7 / 77.8 and 81.0 / 80.3 / 72.3, 9001^2 79.5 / 77.9 / 74.7 and
+  // 79.5 / 76.5 / 71.3; FP16 16384^2, 16 warps of half the bytes, 106.9 / 107.8 /
+  // 107.9)
+  const int most = c->L.storage == 0 && c->L.P_bc == BC_PERIODIC && !c->L.force && P.smodel < 2
+                       ? 32 : 64;
   const double slots = 152 * 15;
   const int strips = march_strips(c->L.P_bc, P.nx);
   double best = 1e300;
   int rows = 16;
   for (int r : {8, 12, 16, 24, 32, 48, 64}) {
+    if (r > most) break;
     const double n = (double)strips * ((P.ny + r - 1) / r);
     const double cost = (n / slots + 1.0) * (r + 3);
     if (cost < best) {
