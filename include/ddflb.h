@@ -232,7 +232,11 @@ ddflb_status ddflb_populations(ddflb_ctx* c, float* f, float* g);
 /* Reduce the current state now and return (synchronising the stream): total
  * mass sum rho, total scalar sum phi, the residual of the last check (NaN if
  * none yet) and the number of steps taken.  Any output pointer may be NULL.
- * Returns EDIVERGED once a non-finite sum has been seen. */
+ * Returns EDIVERGED once a non-finite sum has been seen, ETIMEOUT once a bulk
+ * copy of a step kernel did not arrive in time.  After either the steps leave
+ * the state as it is (after ETIMEOUT it is no state of the lattice) until
+ * ddflb_init or ddflb_set_state; ddflb_fields_host, run_to_tolerance and sums
+ * report ETIMEOUT too, the asynchronous calls cannot. */
 ddflb_status ddflb_stats(ddflb_ctx* c, double* mass, double* scalar, double* residual,
                          int64_t* step);
 /* Advance until steady state (Sec. 5.4 reports the cavity flows at steady
@@ -395,6 +399,8 @@ ddflb_status ddflb_sums(ddflb_ctx* c, int32_t mode, double* out);
 #define DDFLB_INST_CONVERGED 1
 #define DDFLB_INST_DIVERGED 2
 #define DDFLB_INST_CAPPED 4  /* frozen at its own step limit without converging */
+#define DDFLB_INST_LOST 8    /* a bulk copy of a two-step launch did not arrive: frozen, the state
+                              * unusable until ddflb_batch_init (stats, fields: ETIMEOUT) */
 typedef struct ddflb_batch ddflb_batch;
 
 /* Workspace bytes for n instances with parameters p[0..n-1] (0 if invalid). */
@@ -446,7 +452,8 @@ ddflb_status ddflb_batch_fields(ddflb_batch* b, int32_t i, float* rho, float* ux
  * from the instance's last ddflb_batch_init to the check at which the residual
  * first fell below tol (-1: not yet), the state time of its current state and
  * the state time of its last init (so state_time - init_time steps have been
- * run on it).  Synchronises; ETIMEOUT if a barrier wait ran out. */
+ * run on it).  Synchronises; ETIMEOUT if a barrier wait ran out or an instance
+ * is DDFLB_INST_LOST. */
 ddflb_status ddflb_batch_stats(ddflb_batch* b, double* residual, int32_t* flags,
                                int64_t* steps_to_tol, int64_t* state_time, int64_t* init_time);
 /* Autotuner: times every supported tile shape with the persistent launch at

@@ -440,7 +440,7 @@ namespace {
 
 const void* fptr(const ddflb_ctx* c, int buf) { return c->pops[buf]; }
 
-// Zero the device status block (no residual yet, not diverged) on the stream.
+// Zero the device status block (no residual yet, not stopped) on the stream.
 ddflb_status reset_status(ddflb_ctx* c) {
   cudaError_t e = cudaMemsetAsync(c->status, 0, sizeof(DevStatus), c->L.stream);
   return e == cudaSuccess ? DDFLB_OK : cuda_fail(e, "status reset");
@@ -771,7 +771,19 @@ ddflb_status ddflb_fields_host_async(ddflb_ctx* c, float* rho, float* ux, float*
 ddflb_status ddflb_fields_host(ddflb_ctx* c, float* rho, float* ux, float* uy, float* phi,
                                float* sxx, float* sxy, float* syy, float* omega) {
   ddflb_status s = ddflb_fields_host_async(c, rho, ux, uy, phi, sxx, sxy, syy, omega);
-  return s == DDFLB_OK ? ddflb_io_wait(c) : s;
+  DevStatus h{};
+  if (s == DDFLB_OK) {
+    const cudaError_t e =
+        cudaMemcpyAsync(&h, c->status, sizeof h, cudaMemcpyDeviceToHost, c->L.stream);
+    if (e != cudaSuccess) s = cuda_fail(e, "fields_host status");
+  }
+  if (s == DDFLB_OK) s = ddflb_io_wait(c);
+  if (s == DDFLB_OK) {
+    const cudaError_t e = cudaStreamSynchronize(c->L.stream);
+    if (e != cudaSuccess) s = cuda_fail(e, "fields_host");
+  }
+  if (s == DDFLB_OK && (h.stopped & kStopTimeout)) return timed_out(c);
+  return s;
 }
 
 ddflb_status ddflb_io_wait(ddflb_ctx* c) {
@@ -821,8 +833,8 @@ ddflb_status ddflb_stats(ddflb_ctx* c, double* mass, double* scalar, double* res
   if (scalar) *scalar = cells * c->p.phi0 + h.scalar_dev;
   if (residual) *residual = h.has_residual ? h.residual / c->p.check_every : NAN;
   if (step) *step = c->step;
-  if (h.timeout) return timed_out(c);
-  if (h.diverged) return fail(DDFLB_EDIVERGED, "non-finite mass/scalar sum by step %lld",
+  if (h.stopped & kStopTimeout) return timed_out(c);
+  if (h.stopped) return fail(DDFLB_EDIVERGED, "non-finite mass/scalar sum by step %lld",
                               (long long)c->step);
   return DDFLB_OK;
 }
@@ -853,8 +865,8 @@ ddflb_status ddflb_run_to_tolerance(ddflb_ctx* c, double tol, int64_t max_steps,
     cudaError_t e = cudaMemcpyAsync(&h, c->status, sizeof h, cudaMemcpyDeviceToHost, c->L.stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->L.stream);
     if (e != cudaSuccess) return cuda_fail(e, "run_to_tolerance");
-    if (h.timeout) return timed_out(c);
-    if (h.diverged)
+    if (h.stopped & kStopTimeout) return timed_out(c);
+    if (h.stopped)
       return fail(DDFLB_EDIVERGED, "non-finite mass/scalar sum by step %lld", (long long)c->step);
     if (!h.has_residual) continue;  // the first check only takes the snapshot
     const double r = h.residual / K;
@@ -1100,8 +1112,8 @@ ddflb_status ddflb_sums(ddflb_ctx* c, int32_t mode, double* out) {
   out[1] = h.scalar_dev;
   out[2] = h.u2;
   out[3] = (mode & 1) ? h.du2 : NAN;
-  if (h.timeout) return timed_out(c);
-  if (h.diverged) return fail(DDFLB_EDIVERGED, "non-finite sum by step %lld", (long long)c->step);
+  if (h.stopped & kStopTimeout) return timed_out(c);
+  if (h.stopped) return fail(DDFLB_EDIVERGED, "non-finite sum by step %lld", (long long)c->step);
   return DDFLB_OK;
 }
 

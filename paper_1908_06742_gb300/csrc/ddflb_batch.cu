@@ -58,7 +58,7 @@ struct BatchStatus {
   int64_t steps_to_tol;  // state time at which the residual first fell below tol (-1: not yet)
   int64_t state_time;    // state time of the instance's current state when frozen
   long long init_time;   // state time at which the instance was (re)initialised
-  int32_t flags;         // DDFLB_INST_CONVERGED | DDFLB_INST_DIVERGED | DDFLB_INST_CAPPED
+  int32_t flags;         // DDFLB_INST_*: not 0 once frozen
   int32_t buf;           // buffer that holds the state of a frozen instance
   double tol;            // this instance's tolerance (< 0: the batch's)
   int64_t max_steps;     // freeze after this many steps since init (0: no limit)
@@ -458,8 +458,10 @@ __global__ void __launch_bounds__(32, kMarchWarps<S, BC>)
   __syncwarp();
   const S* fin = (const S*)sI.buf[src];
   S* fout = (S*)sI.buf[src ^ 1];
-  march_strip<S, BC>(sI.P, sK, fin, fin + sI.goff, fout, fout + sI.goff, T.y, T.z, T.w,
-                     march_shared, s_bar, s_wall, &A.sync->err);
+  if (!march_strip<S, BC>(sI.P, sK, fin, fin + sI.goff, fout, fout + sI.goff, T.y, T.z, T.w,
+                          march_shared, s_bar, s_wall) &&
+      threadIdx.x == 0)
+    atomicOr(&A.ist[T.x].flags, DDFLB_INST_LOST);  // no step, sum or check of it follows
 }
 
 __global__ void k_batch_advance(BatchSync* sync, int nsteps) {
@@ -825,6 +827,11 @@ cudaGraphExec_t chunk_graph(ddflb_batch* b, int nsteps) {
   return ex;
 }
 
+ddflb_status lost(int i) {
+  return bfail(DDFLB_ETIMEOUT, "a bulk copy of a two-step launch did not arrive: the state of "
+                               "instance %d is lost until it is initialised again", i);
+}
+
 ddflb_status check_sync_error(ddflb_batch* b) {
   BatchSync h;
   cudaError_t e = cudaMemcpyAsync(&h, b->d_sync, sizeof h, cudaMemcpyDeviceToHost, b->stream);
@@ -1050,6 +1057,7 @@ ddflb_status ddflb_batch_fields(ddflb_batch* b, int32_t i, float* rho, float* ux
   cudaError_t e = cudaMemcpyAsync(&s, b->d_status + i, sizeof s, cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bcuda(e, "batch fields status");
+  if (s.flags & DDFLB_INST_LOST) return lost(i);
   const int buf = s.flags ? s.buf : b->cur;
   Launch L;
   L.P = b->lp[i];
@@ -1080,7 +1088,11 @@ ddflb_status ddflb_batch_stats(ddflb_batch* b, double* residual, int32_t* flags,
     if (state_time) state_time[i] = h[i].flags ? h[i].state_time : b->step;
     if (init_time) init_time[i] = h[i].init_time;
   }
-  return check_sync_error(b);
+  const ddflb_status s = check_sync_error(b);
+  if (s != DDFLB_OK) return s;
+  for (int i = 0; i < b->n; ++i)
+    if (h[i].flags & DDFLB_INST_LOST) return lost(i);
+  return DDFLB_OK;
 }
 
 ddflb_status ddflb_batch_debug_skip_barrier(ddflb_batch* b, int32_t block) {

@@ -62,11 +62,13 @@ struct DevStatus {
   double u2;          // sum |u|^2
   double du2;         // sum |u - u_prev|^2 (check reductions)
   double residual;    // sqrt(du2 / u2) of the last check
-  int32_t diverged;   // set once a sum is non-finite
+  int32_t stopped;    // Stop bits; the step kernels leave the state alone once one is set
   int32_t has_residual;
-  int32_t timeout;    // a bulk copy of the two-step kernel did not arrive in time
-  int32_t pad;
+  int64_t pad;
 };
+// a sum is non-finite; a bulk copy of the two-step kernel did not arrive in time, so
+// that part of the state is the one of two steps earlier
+enum Stop : int32_t { kStopDiverged = 1, kStopTimeout = 2 };
 
 // ------------------------------------------------------------ storage codec
 // Loads take the read-only (non-coherent) path by default, for kernels that run

@@ -41,7 +41,7 @@ __global__ void __maxnreg__(56) k_step(LbParams P, const S* __restrict__ fin,
     inner = __all_sync(0xffffffffu, in_x && y >= 1 && y < P.ny - 1);
   }
   if (x >= P.nx || y >= P.y1) return;
-  if (status != nullptr && status->diverged) return;
+  if (status != nullptr && status->stopped) return;
   float df[9], dg[9];
   if (BC != BC_PERIODIC && inner)
     pull<S, BC_PERIODIC>(P, fin, gin, x, y, df, dg);
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(256) k_finalize(const double* __restrict__ par
       st->residual = sh[2][0] > 0.0 ? sqrt(sh[3][0] / sh[2][0]) : 0.0;
       st->has_residual = 1;
     }
-    if (!isfinite(sh[0][0]) || !isfinite(sh[1][0]) || !isfinite(sh[2][0])) st->diverged = 1;
+    if (!isfinite(sh[0][0]) || !isfinite(sh[1][0]) || !isfinite(sh[2][0])) st->stopped |= kStopDiverged;
   }
 }
 

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(128, 5)
   const int nx = P.nx, ny = P.ny;
   const int x0 = 2 * (blockIdx.x * (BX ? BX : blockDim.x) + threadIdx.x);
   const int y = down ? ny - 1 - (int)blockIdx.y : (int)blockIdx.y;
-  if (x0 >= nx || status->diverged) return;
+  if (x0 >= nx || status->stopped) return;
   F2 df[9], dg[9];
   if (BC == BC_PERIODIC || (y >= 1 && y < ny - 1)) {
     const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;

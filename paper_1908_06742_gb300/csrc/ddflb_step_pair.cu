@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) k_step_pair(LbParams P, const S* __restri
   const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (y >= P.ny) return;  // whole warps share y
-  if (status != nullptr && status->diverged) return;
+  if (status != nullptr && status->stopped) return;
   const int nx = P.nx, ny = P.ny;
   const int64_t pl = P.plane;
   const bool live = x0 < nx;
@@ -217,7 +217,7 @@ __global__ void __maxnreg__(96) k_step_quad(LbParams P, const S* __restrict__ fi
   // down: rows in descending order (as k_step_duo)
   const int yb = blockIdx.y * blockDim.y + threadIdx.y, y = down ? P.ny - 1 - yb : yb;
   if (x0 >= P.nx || yb >= P.ny) return;
-  if (status != nullptr && status->diverged) return;
+  if (status != nullptr && status->stopped) return;
   const int nx = P.nx, ny = P.ny;
   const int64_t pl = P.plane;
   if (BC != BC_PERIODIC &&

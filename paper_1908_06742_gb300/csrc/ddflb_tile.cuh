@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(NTH) k_tile(LbParams P, const S* __restrict__ 
   // here, and waits here itself; hence L2-coherent loads below)
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();
-  if (status->diverged) return;
+  if (status->stopped) return;
   const int nx = P.nx, ny = P.ny;
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
   const int x1 = min(x0 + TX, nx), y1 = min(y0 + TY, ny);

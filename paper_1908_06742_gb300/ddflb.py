@@ -161,7 +161,7 @@ SIGNATURES = {
     "ddflb_version": (ctypes.c_char_p, []),
 }
 
-INST_CONVERGED, INST_DIVERGED, INST_CAPPED = 1, 2, 4
+INST_CONVERGED, INST_DIVERGED, INST_CAPPED, INST_LOST = 1, 2, 4, 8
 
 
 def load(path: str = LIB_PATH):
