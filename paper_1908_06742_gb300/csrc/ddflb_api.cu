@@ -941,6 +941,7 @@ ddflb_status ddflb_autotune(ddflb_ctx* c, int32_t trial_steps, int32_t* block_x,
   dim3 bestb(128, 1, 1);
   int bestp = 1;
   const int saved_path = c->path;
+  const dim3 saved_block = c->L.block;
   const size_t gofs = c->lay.gofs;
   for (int pth = 1; pth <= 3 && e == cudaSuccess; ++pth) {
     for (const auto& sh : shapes) {
@@ -1002,11 +1003,11 @@ ddflb_status ddflb_autotune(ddflb_ctx* c, int32_t trial_steps, int32_t* block_x,
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  c->path = saved_path;
-  if (e != cudaSuccess) return cuda_fail(e, "autotune trial");
-  c->L.block = bestb;
-  c->path = bestp;
+  // (with the path and the block go the graphs and what the automatic path chose)
+  c->L.block = e == cudaSuccess ? bestb : saved_block;
+  c->path = e == cudaSuccess ? bestp : saved_path;
   drop_graphs(c);
+  if (e != cudaSuccess) return cuda_fail(e, "autotune trial");
   if (path) *path = bestp;
   e = cudaMemsetAsync(c->pops[0], 0, 2 * c->lay.pops_bytes, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
