@@ -428,8 +428,9 @@ ddflb_status ddflb_batch_set_instance_run(ddflb_batch* b, int32_t i, double tol,
 /* How a chunk of steps is launched: 0 (default) = one persistent cooperative
  * launch with a device-wide barrier between steps; 1 = ordinary launches
  * captured in a graph, the stream as the barrier: two steps per launch between
- * the residual checks (one warp per strip of an instance), single steps with one
- * CTA per tile around them (suits large batches).  Same results bit for bit.
+ * the residual checks where the batch is large enough for it (one warp per strip
+ * of an instance), single steps with one CTA per tile elsewhere (suits large
+ * batches).  Same results bit for bit.
  * The autotuner tries both. */
 ddflb_status ddflb_batch_set_schedule(ddflb_batch* b, int32_t schedule);
 ddflb_status ddflb_batch_get_schedule(const ddflb_batch* b, int32_t* schedule);

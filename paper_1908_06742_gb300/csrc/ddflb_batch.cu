@@ -341,8 +341,8 @@ __global__ void __launch_bounds__(256, 4) k_batch(BatchArgs A) {
 }
 
 // Schedule 1: ordinary launches, ordered by the stream, captured in one graph
-// per chunk: two steps per launch (k_batch_march) between the check steps, and
-// around them single steps (k_batch_tile, one CTA per tile), each check step
+// per chunk: two steps per launch (k_batch_march) between the check steps where that
+// is faster (two_steps_pay), and around them single steps (k_batch_tile, one CTA per tile), each check step
 // followed by the sums and the check.  Step s of the chunk advances the state
 // from time sync->step + s.  The node update carries no check code; at most 56
 // registers, so 9 CTAs of 128 threads stay resident.
@@ -504,12 +504,36 @@ struct BLayout {
   int max_tiles;
   int item_rows;        // rows per item of the two-step launches
   int item_begin[4];    // items by boundary kind: [item_begin[bc], item_begin[bc + 1])
+  bool two_steps;       // schedule 1 takes two steps per launch between the checks
 };
 
 int count_tiles(int n, const ddflb_params* p, int tx, int ty) {
   int64_t t = 0;
   for (int i = 0; i < n; ++i) t += (int64_t)((p[i].nx + tx - 1) / tx) * ((p[i].ny + ty - 1) / ty);
   return t > (1 << 30) ? -1 : (int)t;
+}
+
+// Whether two steps per launch are faster than one, from `items` warps that take
+// `rows` rows' time: a small batch has too few strips, and lattices of 64 or 128
+// columns leave lanes of the 64-column strips without a node.  us per step, one step
+// per launch, two (72 batches of 4 to 256 lattices of 64^2 to 512^2: the choice is
+// within 5 % of the better one, but for 6 x 400^2 FP32 periodic 29.0, 26.7):
+//   FP32 cavities   4 x 64^2 3.0, 13.4   8 x 256^2 14.3, 20.4   32 x 256^2 61.0, 56.3
+//   FP32 periodic   256 x 64^2 31.2, 48.9   128 x 128^2 59.9, 67.3   8 x 512^2 56.7, 51.4
+//   BF16 cavities   256 x 128^2 101, 119   256 x 64^2 26.0, 25.5   8 x 512^2 49.2, 46.8
+//   BF16 periodic   16 x 256^2 22.4, 27.2   4 x 512^2 22.4, 21.1   16 x 512^2 89.7, 69.2
+bool two_steps_pay(int n, const ddflb_params* p, int64_t items, double rows) {
+  double knodes = 0.0;
+  bool walls = false;
+  for (int i = 0; i < n; ++i) {
+    knodes += 1e-3 * p[i].nx * p[i].ny;
+    walls = walls || p[i].bc != DDFLB_BC_PERIODIC;
+  }
+  const bool fp32 = p[0].storage == DDFLB_FP32;
+  // us per row (and step); 16-bit items of one wave of 16 warps an SM have the FP32
+  // units nearly to themselves
+  const double row = !fp32 && items <= 152 * 16 ? 1.0 : fp32 || walls ? 1.3 : 1.1;
+  return row * rows < 3.0 + (fp32 ? 0.0275 : 0.0228) * knodes;
 }
 
 BLayout blayout(int n, const ddflb_params* p) {
@@ -537,7 +561,7 @@ BLayout blayout(int n, const ddflb_params* p) {
     for (int i = 0; i < n; ++i) k += (int64_t)march_strips(p[i].bc, p[i].nx) * ((p[i].ny + r - 1) / r);
     return k;
   };
-  double best = 1e300;
+  double best = 1e300;  // in rows
   for (int r : {8, 12, 16, 24, 32, 48, 64}) {
     const double cost = ((double)items(r) / (152 * 12) + 1.0) * (r + 3);
     if (cost < best) {
@@ -545,6 +569,7 @@ BLayout blayout(int n, const ddflb_params* p) {
       L.item_rows = r;
     }
   }
+  L.two_steps = two_steps_pay(n, p, items(L.item_rows), best);
   L.off_items = o; o += al((size_t)items(L.item_rows) * sizeof(int4));
   L.off_consts = o; o += al(n * sizeof(PairConst));
   L.total = o;
@@ -740,7 +765,7 @@ cudaError_t launch_chunk(ddflb_batch* b, cudaStream_t s, int nsteps, int64_t t0,
     for (int k = 0; k < nsteps; cur ^= 1) {
       const int64_t t = t0 + k;
       cudaError_t e;
-      if (k + 1 < nsteps && !check_at(t) && !check_at(t + 1)) {
+      if (b->lay.two_steps && k + 1 < nsteps && !check_at(t) && !check_at(t + 1)) {
         e = b->storage == 0   ? launch_two<float>(b, s, A, cur)
             : b->storage == 1 ? launch_two<__half>(b, s, A, cur)
                               : launch_two<__nv_bfloat16>(b, s, A, cur);
@@ -789,7 +814,7 @@ int chunk_end(const ddflb_batch* b, int nsteps) {
   auto check_at = [&](int64_t t) { return K > 0 && t % K == 0; };
   for (int k = 0; k < nsteps; cur ^= 1) {
     const int64_t t = b->step + k;
-    k += k + 1 < nsteps && !check_at(t) && !check_at(t + 1) ? 2 : 1;
+    k += b->lay.two_steps && k + 1 < nsteps && !check_at(t) && !check_at(t + 1) ? 2 : 1;
   }
   return cur;
 }
