@@ -168,7 +168,10 @@ ddflb_status ddflb_init_host(ddflb_ctx* c, const float* rho, const float* ux, co
  * r = |u(t) - u(t-K)|_2 / (K |u(t)|_2) (FP64 sums; the mean relative change
  * per step over the interval, which stays above the FP32 rounding jitter of a
  * one-step difference) in the device status block; once a sum is non-finite
- * further steps are skipped and the next ddflb_stats returns EDIVERGED. */
+ * further steps are skipped and the next ddflb_stats returns EDIVERGED.
+ * On a stream that the caller is capturing, an even n advances the state at every
+ * replay of the graph (one step per launch); step counts that the library reports
+ * and a lattice's residual checks follow the calls, not the replays. */
 ddflb_status ddflb_step(ddflb_ctx* c, int64_t n);
 
 /* Local kinematics of the current state (Sec. 4): density, velocity, scalar,
@@ -444,7 +447,8 @@ ddflb_status ddflb_batch_get_tiles(const ddflb_batch* b, int32_t* tile_x, int32_
  * ddflb_init (clears its converged/diverged flags). */
 ddflb_status ddflb_batch_init(ddflb_batch* b, int32_t i, const float* rho, const float* ux,
                               const float* uy, const float* phi, const float* grads);
-/* Advance all active instances n steps (asynchronous). */
+/* Advance all active instances n steps (asynchronous).  Captured by the caller:
+ * as ddflb_step. */
 ddflb_status ddflb_batch_step(ddflb_batch* b, int64_t n);
 /* Local kinematics of instance i's current state, as ddflb_fields. */
 ddflb_status ddflb_batch_fields(ddflb_batch* b, int32_t i, float* rho, float* ux, float* uy,

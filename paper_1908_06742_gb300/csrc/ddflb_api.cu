@@ -663,8 +663,9 @@ ddflb_status ddflb_step(ddflb_ctx* c, int64_t n) {
     c->march_rows = choose_march_rows(c);
     c->tile = choose_tile(c);
   }
+  const bool single = capturing(c->L.stream);  // one step per launch, no graph of our own
   while (n > 0) {
-    if (c->p.force_omega == 0.0 && !c->graph_failed) {
+    if (!single && c->p.force_omega == 0.0 && !c->graph_failed) {
       // whole graphs up to the next check step (checks run after it, as below)
       const int64_t until = K > 0 ? std::min<int64_t>(n, K - c->step % K) : n;
       const int64_t reps = until / kGraphSteps;
@@ -683,7 +684,7 @@ ddflb_status ddflb_step(ddflb_ctx* c, int64_t n) {
         continue;
       }
     }
-    if (n > 1 && c->march_rows > 0 && (K == 0 || K - c->step % K >= 2)) {
+    if (!single && n > 1 && c->march_rows > 0 && (K == 0 || K - c->step % K >= 2)) {
       cudaError_t e = run_two(c, c->cur);
       if (e != cudaSuccess) return cuda_fail(e, "step");
       c->cur ^= 1;
@@ -694,7 +695,7 @@ ddflb_status ddflb_step(ddflb_ctx* c, int64_t n) {
       continue;
     }
     constexpr int T = kTileSteps;
-    if (c->tile >= 0 && n >= T && (K == 0 || K - c->step % K >= T)) {
+    if (!single && c->tile >= 0 && n >= T && (K == 0 || K - c->step % K >= T)) {
       cudaError_t e = run_tile(c, c->cur);
       if (e != cudaSuccess) return cuda_fail(e, "step");
       c->cur ^= 1;

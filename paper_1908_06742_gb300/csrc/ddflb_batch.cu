@@ -386,6 +386,7 @@ __global__ void __launch_bounds__(256) k_batch_sums(BatchArgs A, int s, int src)
   __shared__ int sActive;
   __shared__ long long sInit;
   const int64_t t = A.sync->step + s;
+  if (t % A.check_every != 0) return;  // (a caller's graph launches it after every step)
   const LbParams& sP = sI.P;
   const int tx = threadIdx.x % A.tile_x, ty = threadIdx.x / A.tile_x;
   int cur = -1;
@@ -432,7 +433,9 @@ __global__ void __launch_bounds__(256) k_batch_sums(BatchArgs A, int s, int src)
 // K): one CTA per instance.
 __global__ void __launch_bounds__(256) k_batch_check(BatchArgs A, int s, int dst) {
   __shared__ double sh[8];
-  check_instance(A, blockIdx.x, A.sync->step + s, dst, sh);
+  const int64_t t = A.sync->step + s;
+  if (t == 0 || t % A.check_every != 0) return;  // (as k_batch_sums)
+  check_instance(A, blockIdx.x, t, dst, sh);
 }
 
 // Two steps of every active instance: one warp per item (instance, strip, rows),
@@ -752,8 +755,11 @@ cudaError_t launch_two(ddflb_batch* b, cudaStream_t s, const BatchArgs& A, int s
 }
 
 // One chunk of nsteps steps from state time t0 and buffer b->cur; *end: the
-// buffer of the state after it.
-cudaError_t launch_chunk(ddflb_batch* b, cudaStream_t s, int nsteps, int64_t t0, int* end) {
+// buffer of the state after it.  replayed: into a caller's graph, whose replays start
+// at other state times: single steps, each followed by the sums and the check, which
+// look at the time on the device.
+cudaError_t launch_chunk(ddflb_batch* b, cudaStream_t s, int nsteps, int64_t t0, int* end,
+                         bool replayed = false) {
   BatchArgs A = args_for(b, nsteps);
   if (b->schedule == 1) {
     const dim3 tb(b->tile_x * b->tile_y);
@@ -765,7 +771,7 @@ cudaError_t launch_chunk(ddflb_batch* b, cudaStream_t s, int nsteps, int64_t t0,
     for (int k = 0; k < nsteps; cur ^= 1) {
       const int64_t t = t0 + k;
       cudaError_t e;
-      if (b->lay.two_steps && k + 1 < nsteps && !check_at(t) && !check_at(t + 1)) {
+      if (b->lay.two_steps && !replayed && k + 1 < nsteps && !check_at(t) && !check_at(t + 1)) {
         e = b->storage == 0   ? launch_two<float>(b, s, A, cur)
             : b->storage == 1 ? launch_two<__half>(b, s, A, cur)
                               : launch_two<__nv_bfloat16>(b, s, A, cur);
@@ -776,10 +782,10 @@ cudaError_t launch_chunk(ddflb_batch* b, cudaStream_t s, int nsteps, int64_t t0,
       void* targs[] = {&A, &cur};
       e = cudaLaunchKernel(batch_kernel(b->storage, 1, b->bcs), dim3(b->ntiles), tb, targs, 0, s);
       if (e != cudaSuccess) return e;
-      if (check_at(t)) {  // (t = 0: the first snapshot)
+      if (check_at(t) || (replayed && K > 0)) {  // (t = 0: the first snapshot)
         void* sargs[] = {&A, &k, &cur};
         e = cudaLaunchKernel(sums, dim3(b->sums_grid), tb, sargs, 0, s);
-        if (e == cudaSuccess && t > 0) {
+        if (e == cudaSuccess && (t > 0 || replayed)) {
           k_batch_check<<<b->n, 256, 0, s>>>(A, k, cur ^ 1);
           e = cudaGetLastError();
         }
@@ -1073,13 +1079,14 @@ ddflb_status ddflb_batch_step(ddflb_batch* b, int64_t n) {
   struct PopRange {
     ~PopRange() { nvtxRangePop(); }
   } pop_range;
+  const bool replayed = capturing(b->stream);
   int64_t left = n;
   while (left > 0) {
     const int k = (int)std::min<int64_t>(left, b->chunk);
-    cudaGraphExec_t ex = k == b->chunk ? chunk_graph(b, k) : nullptr;
+    cudaGraphExec_t ex = k == b->chunk && !replayed ? chunk_graph(b, k) : nullptr;
     int end = chunk_end(b, k);
-    const cudaError_t e =
-        ex ? cudaGraphLaunch(ex, b->stream) : launch_chunk(b, b->stream, k, b->step, &end);
+    const cudaError_t e = ex ? cudaGraphLaunch(ex, b->stream)
+                             : launch_chunk(b, b->stream, k, b->step, &end, replayed);
     if (e != cudaSuccess) return bcuda(e, "batch step launch");
     left -= k;
     b->step += k;

@@ -14,6 +14,17 @@ inline int march_strips(int bc, int nx) {
   if (bc == BC_CAVITY) return nx <= 64 ? 1 : 1 + (nx - 64 + kMarchStrip - 1) / kMarchStrip;
   return (nx + kMarchStrip - 1) / kMarchStrip;
 }
+// Whether the caller is capturing the stream into a graph of its own.  The host
+// keeps track of the buffer that holds the state, and replays do not pass through
+// it: what is captured has to end where single steps would, so that an even number
+// of steps advances the state at every replay.
+inline bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // (the legacy stream beside another one's capture)
+  return false;
+}
+
 constexpr int kMaxGridY = 65535;  // blocks of a grid in y
 constexpr int kReduceThreads = 256;
 constexpr int kReduceBlocks = 608;  // 4 per SM on a 152-SM GB300; fixed for deterministic sums
