@@ -539,7 +539,8 @@ ddflb_status ddflb_nn_set_conv_path(int32_t path);
  * tile fits shared memory (W a multiple of 128, or up to 250 and more where C
  * is small; else EINVAL): each tile of 128 positions is copied once with its
  * halo and read by all nine taps.  Bit-identical to im2col + ddflb_nn_gemm.
- * ddflb_nn_conv3x3 takes this form for C = 64 on path 0. */
+ * ddflb_nn_conv3x3 takes this form for C = 64 on path 0, except for FP32
+ * output of few pixels. */
 ddflb_status ddflb_nn_conv3x3_narrow(const void* X, int32_t B, int32_t H, int32_t W, int32_t C,
                                      int32_t cs, const void* Wt, int32_t N, float* Cf, int32_t ldc,
                                      void* Cb, int32_t ldcb, const float* bias, int32_t act,

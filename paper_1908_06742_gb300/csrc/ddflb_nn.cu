@@ -1606,6 +1606,22 @@ bool narrow_fits(int B, int H, int W, int C, int N, int bn) {
   return narrow_args(&a, nullptr, B, H, W, C, C, nullptr, bn, 1, g);
 }
 
+// Whether 64 channels go through the narrow kernel rather than the TMA boxes: always
+// with BF16 output, but FP32 rows fill its epilogue, and its outputs come in tiles of
+// 64 (the boxes: 128), so there the boxes are faster while they take a wave or two and
+// it takes more.  us, boxes and narrow, FP32 output, 16 images:
+//   32^2 N 64 10.5, 12.5   N 96 12.6, 18.7   N 128 12.6, 16.7   N 256 18.7, 20.7
+//   64^2 N 64 21.4, 18.6   N 96 31.0, 28.9   N 128 30.1, 26.8   N 256 47.5, 45.3
+//   128^2 N 64 57.7, 45.5  N 128 87.6, 82.7  (4 images: N 96 31.0, 32.9)
+// (BF16: 32^2 N 128 14.6, 14.6; 64^2 32.1, 22.9; 128^2 91.7, 65.6.)
+bool narrow_pays(int64_t P, int W, int N, bool fp32) {
+  if (!fp32) return true;
+  const int64_t sm = sm_count(), t = (P + 127) / 128;
+  if (N <= 64) return t > sm || (N <= 32 ? 2 : 4) * t <= sm;
+  const int waves = N % 128 != 0 && N > 128 ? 1 : N < 128 && W % 128 == 0 ? 4 : 2;
+  return t * ((N + 63) / 64) <= sm || t * ((N + 127) / 128) > waves * sm;
+}
+
 // The channels that the weight gradient takes, and the images: positions are
 // divided by the padded rows' length with one 32-bit multiplication.
 bool wgrad_channels(int Ci, int Co) {
@@ -1805,7 +1821,7 @@ ddflb_status ddflb_nn_conv3x3(const void* X, int32_t B, int32_t H, int32_t W, in
   g.conv_bh = bh;
   g.conv_bb = bb;
   cudaStream_t s = (cudaStream_t)stream;
-  if (C == 64 && g_conv_path == 0) {
+  if (C == 64 && g_conv_path == 0 && narrow_pays((int64_t)B * H * W, W, N, Cf != nullptr)) {
     bool refused;
     const ddflb_status st = narrow_fwd<8>(X, B, H, W, cs, Wt, g, s, &refused);
     if (!refused) return st;
