@@ -636,7 +636,7 @@ ddflb_status ddflb_warm_fields(const float* pred, int32_t nx, int32_t ny, int32_
 /* Message of the last error on the calling thread ("" if none). */
 const char* ddflb_last_error(void);
 
-/* Library version string. */
+/* Library version string; a tuning found with another version is not this one's. */
 const char* ddflb_version(void);
 
 #ifdef __cplusplus

@@ -922,7 +922,9 @@ ddflb_status ddflb_destroy(ddflb_ctx* c) {
 
 const char* ddflb_last_error(void) { return g_err.c_str(); }
 
-const char* ddflb_version(void) { return "ddflb 0.1 (sm_103a)"; }
+// (part of the key of cached tunings: a new one whenever kernels or the rules between
+// them change what an autotuner measured)
+const char* ddflb_version(void) { return "ddflb 0.2 (sm_103a)"; }
 
 // Autotuner for the step kernel's block shape: each candidate runs trial_steps
 // untimed, then trial_steps timed with CUDA events on the context stream; the

@@ -1,8 +1,8 @@
 """JSON cache of autotuner choices (tile shapes, block shapes, residency).
 
-Keyed by device name, the kind of launch, storage precision and a digest of
-the instance sizes, so a tuning found once is reused on the same GPU model for
-the same workload shape.  File: $DDFLB_TUNE_CACHE or ~/.cache/ddflb/tuning.json.
+Keyed by device name, library version, the kind of launch, storage precision and
+a digest of the instance sizes, so a tuning found once is reused on the same GPU
+model for the same workload shape, until the kernels that it chose from change.  File: $DDFLB_TUNE_CACHE or ~/.cache/ddflb/tuning.json.
 """
 from __future__ import annotations
 
@@ -24,10 +24,15 @@ def _device() -> str:
         return "unknown"
 
 
+def _version() -> str:
+    from . import ddflb
+    return ddflb.load().ddflb_version().decode()
+
+
 def key(kind: str, cfgs) -> str:
     sizes = ",".join(f"{c.nx}x{c.ny}:{c.bc}" for c in cfgs)
     digest = hashlib.sha256(sizes.encode()).hexdigest()[:16]
-    return f"{_device()}|{kind}|{cfgs[0].storage}|n={len(cfgs)}|{digest}"
+    return f"{_device()}|{_version()}|{kind}|{cfgs[0].storage}|n={len(cfgs)}|{digest}"
 
 
 def _load() -> dict:
