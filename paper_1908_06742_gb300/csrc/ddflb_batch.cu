@@ -1176,6 +1176,7 @@ ddflb_status ddflb_batch_autotune(ddflb_batch* b, int32_t trial_steps, int32_t* 
   int bx = 128, by = 1, bb = 0, bs = 0;
   ddflb_status rs = DDFLB_OK;
   const int saved_schedule = b->schedule;
+  trial_steps = std::max(trial_steps, 2);  // (what schedule 1 launches between two checks)
   // candidates per tile shape: the persistent launch at full and half
   // residency (variant 0, 1), and one launch per step (variant 2)
   for (int k = 0; k < kNumShapes && rs == DDFLB_OK; ++k) {
