@@ -290,8 +290,10 @@ __device__ __forceinline__ void tma_4d(uint32_t dst, const CUtensorMap* map, int
 #define DDFLB_R8(i) "=r"(r[i]), "=r"(r[i + 1]), "=r"(r[i + 2]), "=r"(r[i + 3]), \
                     "=r"(r[i + 4]), "=r"(r[i + 5]), "=r"(r[i + 6]), "=r"(r[i + 7])
 
-// 32 consecutive FP32 columns of the calling thread's tensor-memory lane
+// 32 consecutive FP32 columns of the calling thread's tensor-memory lane (by the whole
+// warp together: lanes that skipped the last rows' stores join the others first)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32]) {
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
       "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
