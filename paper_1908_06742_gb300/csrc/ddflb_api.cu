@@ -251,6 +251,17 @@ int64_t duo_min_nodes(const Launch& L) {
   return L.force || L.P.smodel >= 2 ? 20000 : 0;
 }
 
+// Rows too narrow for two nodes per thread: at most 32 columns are one warp either way,
+// of half the lanes with twice the work, and the second of two warps of 33 to 48 pairs
+// is nearly empty, which tells while the lattice is small.  us per step, one node -> two:
+// FP32 periodic 20 x 20000 16.3 -> 18.9, 32 x 12500 10.0 -> 12.0, 34 x 11764 17.5 -> 14.1,
+// 66 x 6060 11.9 -> 12.5, 96 x 4166 8.3 -> 8.5, 96 x 16666 37.6 -> 35.8; BF16 8 x 50000
+// 36.3 -> 40.6 (four nodes 77.6).
+bool narrow_rows(const Launch& L, int64_t nodes) {
+  const int nx = L.P.nx;
+  return nx <= 32 || (L.storage == 0 && nx > 64 && nx <= 96 && nodes < 1000000);
+}
+
 cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void* fout, void* gout) {
   const bool whole = c->L.P.y0 == 0 && c->L.P.y1 == c->L.P.ny;
   const int64_t nodes = (int64_t)c->L.P.nx * c->L.P.ny;
@@ -261,11 +272,12 @@ cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void*
   // k_step_duo instead cost its other lattices up to 1 %: 1023 x 767 FP16 1940 ->
   // 1959 us per 200 steps.)
   const bool tall = c->path == 0 && c->L.P.ny > kMaxGridY;
-  const bool quad = quad_step_eligible(c->L) && !tall;
+  const bool narrow = c->path == 0 && whole && narrow_rows(c->L, nodes);
+  const bool quad = quad_step_eligible(c->L) && !tall && !narrow;
   // two nodes per thread in packed arithmetic (unforced MRT 16-bit periodic lattices:
   // until the four-node kernel's wider accesses pay; 1024^2 11.65 us per step
   // against 12.0, 700^2 7.65 against 6.8)
-  if (c->path == 0 && whole && !tall && nodes >= duo_min_nodes(c->L) &&
+  if (c->path == 0 && whole && !tall && !narrow && nodes >= duo_min_nodes(c->L) &&
       !(quad && c->L.P_bc == BC_PERIODIC && nodes > 900000)) {
     auto* launch = c->L.storage == 0   ? launch_step_duo_f32
                    : c->L.storage == 1 ? launch_step_duo_f16
