@@ -235,7 +235,7 @@ namespace ddflb {
 bool pair_step_eligible(const Launch& L);
 cudaError_t launch_step_pair(const Launch& L, const void* fin, const void* gin, void* fout,
                              void* gout, const DevStatus* st);
-// periodic 16-bit lattices with nx a multiple of 4: four nodes per thread
+// 16-bit lattices with nx a multiple of 4: four nodes per thread
 bool quad_step_eligible(const Launch& L);
 cudaError_t launch_step_quad(const Launch& L, const void* fin, const void* gin, void* fout,
                              void* gout, const DevStatus* st, bool down);
@@ -262,6 +262,16 @@ bool narrow_rows(const Launch& L, int64_t nodes) {
   return nx <= 32 || (L.storage == 0 && nx > 64 && nx <= 96 && nodes < 1000000);
 }
 
+// Where four nodes per thread are faster than two (16-bit storage, eligible lattices),
+// up to the two-step kernel.  us per step, two -> four: periodic 1024^2 FP16 12.0 ->
+// 11.7, 700^2 6.8 -> 7.7; channel FP16 1600^2 34.0 -> 34.5, 2000^2 52.2 -> 48.9, 8192 x
+// 700 73.6 -> 68.4.  A cavity's groups at the ends of a row step node by node: FP16
+// 2048^2 56.1 -> 64.9, 16000 x 250 54.7 -> 50.9.
+bool quad_pays(const Launch& L, int64_t nodes) {
+  if (L.P_bc == BC_PERIODIC) return nodes > 900000;
+  return nodes >= 3000000 && (L.P_bc == BC_CHANNEL || L.P.nx >= 8192);
+}
+
 cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void* fout, void* gout) {
   const bool whole = c->L.P.y0 == 0 && c->L.P.y1 == c->L.P.ny;
   const int64_t nodes = (int64_t)c->L.P.nx * c->L.P.ny;
@@ -274,11 +284,9 @@ cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void*
   const bool tall = c->path == 0 && c->L.P.ny > kMaxGridY;
   const bool narrow = c->path == 0 && whole && narrow_rows(c->L, nodes);
   const bool quad = quad_step_eligible(c->L) && !tall && !narrow;
-  // two nodes per thread in packed arithmetic (unforced MRT 16-bit periodic lattices:
-  // until the four-node kernel's wider accesses pay; 1024^2 11.65 us per step
-  // against 12.0, 700^2 7.65 against 6.8)
+  // two nodes per thread in packed arithmetic
   if (c->path == 0 && whole && !tall && !narrow && nodes >= duo_min_nodes(c->L) &&
-      !(quad && c->L.P_bc == BC_PERIODIC && nodes > 900000)) {
+      !(quad && quad_pays(c->L, nodes))) {
     auto* launch = c->L.storage == 0   ? launch_step_duo_f32
                    : c->L.storage == 1 ? launch_step_duo_f16
                                        : launch_step_duo_bf16;
