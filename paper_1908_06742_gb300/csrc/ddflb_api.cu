@@ -308,13 +308,15 @@ cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void*
 // kernel: FP32 periodic 1100^2 26.7 / 25.4, 1200^2 28.6 / 29.1, 2048^2 68 / 84;
 // FP32 cavity 1200^2 31.5 / 29.5, 1400^2 39.3 / 39.9; 16-bit cavity 2048^2 58.5 /
 // 56.1, 4096^2 210 / 246; 16-bit periodic 2048^2 54.3 / 49.3 (four nodes per
-// thread), 4096^2 180 / 186.  FP32 with a uniform force 1450^2 44.8 / 44.8, 2048^2
-// 78 / 85; forced cascaded 2048^2 93 / 88, 4096^2 322 / 351, 8192 x 4096 605 / 703.
+// thread), 4096^2 180 / 186; channel 2500^2 81.4 / 77.7.  FP32 with a uniform force
+// 1450^2 44.8 / 44.8, 2048^2 78 / 85; forced cascaded 2048^2 93 / 88, 4096^2 322 /
+// 351, 8192 x 4096 605 / 703.
 int64_t march_min_nodes(const Launch& L) {
   if (L.P.smodel >= 2) return 10000000;
   if (L.force) return 3000000;
   if (L.storage == 0) return L.P_bc == BC_PERIODIC ? 1400000 : 2000000;
-  return quad_step_eligible(L) && L.P_bc == BC_PERIODIC ? 10000000 : 6000000;
+  if (!quad_step_eligible(L) || L.P_bc == BC_CAVITY) return 6000000;
+  return L.P_bc == BC_PERIODIC ? 10000000 : 8000000;
 }
 
 // Rows per warp of the two-step kernel (ddflb_march.cuh), or 0 where steps go
@@ -327,7 +329,16 @@ int choose_march_rows(const ddflb_ctx* c) {
   if ((c->L.force || P.smodel >= 2) &&
       (c->L.storage != 0 || P.ffield != nullptr || c->p.force_omega != 0.0))
     return 0;
-  if ((int64_t)P.nx * P.ny < march_min_nodes(c->L)) return 0;
+  const int strips = march_strips(c->L.P_bc, P.nx);
+  // Lanes of the 64-column strips without a node of their own cost the two-step kernel
+  // as much as the others, so the line lies higher where few columns leave many.  us
+  // per step, the best single-step kernel, two steps per launch: FP32 periodic 64 x
+  // 25000 31.7, 54.8, 64 x 62500 81.6, 124, 128 x 12500 31.8, 43.0, 184 x 8695 33.2,
+  // 38.6, 184 x 21739 82.8, 85.5, 180 x 8888 37.4, 35.6; cavity 128 x 31250 84.0, 105;
+  // BF16 channel 128 x 62500 103, 159, 256 x 46875 154, 185, 300 x 26666 117, 113.
+  const double filled = (double)P.nx / (64.0 * strips);
+  const double line = filled >= 0.85 ? 1.0 : filled >= 0.7 && c->L.storage == 0 ? 2.2 : 4.0;
+  if ((double)P.nx * P.ny < line * march_min_nodes(c->L)) return 0;
   // strips x chunks in waves of 15 warps an SM, plus most of a chunk at the end
   // while the last ones finish (FP32 8192^2, rows 16 / 32 / 64 / 128: 878, 853,
   // 870, 1023 us per step; 4096^2: 231, 237, 261, 325).  The periodic FP32 form,
@@ -341,7 +352,6 @@ int choose_march_rows(const ddflb_ctx* c) {
   const int most = c->L.storage == 0 && c->L.P_bc == BC_PERIODIC && !c->L.force && P.smodel < 2
                        ? 32 : 64;
   const double slots = 152 * 15;
-  const int strips = march_strips(c->L.P_bc, P.nx);
   double best = 1e300;
   int rows = 16;
   for (int r : {8, 12, 16, 24, 32, 48, 64}) {
