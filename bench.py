@@ -62,8 +62,9 @@ def parse():
                     help="surrogate: training draws run from rest before a first network "
                          "warm-starts the remaining ones (0: all from rest)")
     ap.add_argument("--conv-path", type=int, default=0, choices=[0, 1],
-                    help="conv workload: 0 halo bands where W is a multiple of 128 and C >= 128, "
-                         "1 one box per tap everywhere")
+                    help="conv workload: 0 the narrow kernel for 64 channels, TMA boxes (halo "
+                         "bands where W is a multiple of 128) for more; 1 one TMA box per tap "
+                         "everywhere")
     ap.add_argument("--gemm-shape", default=None,
                     help="gemm workload: one M,N,K,splits shape instead of the U-Net set")
     return ap.parse_args()
@@ -981,8 +982,8 @@ CONV_SHAPES = [(256, 256, 64, 32), (128, 128, 64, 64), (128, 128, 128, 64), (128
 
 
 def run_conv(args, world, rank, local):
-    """The surrogate's 3x3 convolutions: implicit GEMM on tcgen05 (4-D TMA
-    boxes per tap, no patch matrix) against im2col + the tcgen05 GEMM, CUDA
+    """The surrogate's 3x3 convolutions: implicit GEMM on tcgen05 (64 channels
+    from planes copied once, more through 4-D TMA boxes; no patch matrix) against im2col + the tcgen05 GEMM, CUDA
     events per shape; reports the aggregate BF16 TFLOP/s of the implicit form
     and the DRAM-free bound of each (2 P N 9 C flops)."""
     import torch
@@ -1064,8 +1065,8 @@ def run_conv(args, world, rank, local):
         "data": "synthetic",
         "config": {"workload": "U-Net 3x3 convolutions with >= 64 input channels, 256^2 level "
                                "sizes, batch 16, forward (BF16 out, leaky ReLU)",
-                   "kernel": "implicit GEMM, tcgen05 + 4-D TMA (ddflb_nn_conv3x3) vs im2col + "
-                             "tcgen05 GEMM"},
+                   "kernel": "implicit GEMM on tcgen05 (ddflb_nn_conv3x3: k_conv_narrow for 64 "
+                             "channels, 4-D TMA boxes for more) vs im2col + tcgen05 GEMM"},
         "roofline": {"bound": "tensor", "achieved": round(agg["implicit"], 1), "peak": peak,
                      "unit": "TFLOP/s", "frac": round(agg["implicit"] / peak, 4), "peak_kind": kind,
                      # the layers' own roofline: sum over shapes of max(tensor time, HBM

@@ -311,10 +311,11 @@ ddflb_status ddflb_set_block(ddflb_ctx* c, int32_t block_x, int32_t block_y);
  * 2, then 1);
  * 0 (default) = by size: four steps per launch on small lattices (about 256^2
  * at most, no time-dependent force), two on large ones (from 1.4 to 10 million
- * nodes on, no force field; 16-bit storage: MRT or SRT, no force), single steps
- * with two nodes per thread between them and where a call or a residual check
- * leaves some (16-bit periodic ones of a million nodes with four).  All give bit-identical
- * results; which is faster depends on the shape, so the autotuner times them. */
+ * nodes on, more where a row has few columns; no force field; 16-bit storage: MRT
+ * or SRT, no force), single steps with two nodes per thread between them and where
+ * a call or a residual check leaves some (with four on larger 16-bit lattices, with
+ * one on rows of at most 32 columns).  All give bit-identical results; which is
+ * faster depends on the shape, so the autotuner times them. */
 ddflb_status ddflb_set_path(ddflb_ctx* c, int32_t path);
 
 /* Spatially varying part of the body force (Sec. 2; e.g. the four-rolls mill

@@ -1,8 +1,9 @@
 // One time step with two adjacent nodes per thread and packed FP32 arithmetic
 // (k_step_duo), for the lattices between those that take four steps per launch
-// and those that take two, and for those with a force or a central-moment
-// scalar model, which those kernels do not serve (which kernel where:
-// ddflb_api.cu).
+// and those that take two, and above the four-step kernel's at any size for what
+// the two-step kernel does not serve: force fields, time-dependent forces, and
+// 16-bit storage with a force or a central-moment scalar model (which kernel
+// where: ddflb_api.cu).
 #pragma once
 
 #include <cuda_runtime.h>

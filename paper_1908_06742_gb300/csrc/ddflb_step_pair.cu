@@ -13,9 +13,9 @@
 // bit-identical to the one-node kernel.
 //
 // Requirements: nx even (k_step_pair), nx a multiple of 4 (k_step_quad).  By
-// default k_step_quad steps periodic lattices of a million nodes (1024^2 FP16 11.7 us
-// per step, two nodes per thread in packed arithmetic 12.0); k_step_pair runs on
-// an explicit path only.
+// default k_step_quad steps the lattices where it is faster than two nodes per
+// thread in packed arithmetic (quad_pays in ddflb_api.cu); k_step_pair runs on an
+// explicit path, and on periodic lattices of more than 65535 rows.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>

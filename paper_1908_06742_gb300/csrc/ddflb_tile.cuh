@@ -15,9 +15,11 @@ namespace ddflb {
 // that CTAs need nothing from each other within a launch; levels 1 .. T - 1
 // stay in shared memory (two buffers, read and written in turn).
 //
-// A small lattice is bound by the launch and by the latency of one node's
-// update (about 0.5 us), not by any rate: one step per launch takes 2.0 us at
-// 64^2 FP32, four per launch 0.90 us a step, the redundant nodes included
+// A small lattice is bound by the launch and by the length of one thread's
+// instruction stream (about 520 instructions a node and level; 64^2: five warps on
+// the four schedulers at the first level), not by any rate; the largest tile, 32 x
+// 14, has 24 to 14 warps a level and spends more than half of a launch on issue.
+// One step per launch takes 2.0 us at 64^2 FP32, four per launch 0.90 us a step, the redundant nodes included
 // (128^2 cavity 2.2 -> 1.16, 256^2 cavity 3.2 -> 2.1, periodic BF16 2.5 -> 1.6;
 // cascaded 64^2 2.1 -> 1.12, central moments 2.0 -> 0.87, cascaded with a force
 // 256^2 cavity 3.5 -> 2.9).
