@@ -348,7 +348,8 @@ int choose_march_rows(const ddflb_ctx* c) {
   // 48 / 64 rows: 16384^2 81.4 / 81.8 / 80.0 on one, 81.4 / 81.4 / 72.0 on another,
   // 12288^2 81.0 / 80.7 / 77.8 and 81.0 / 80.3 / 72.3, 9001^2 79.5 / 77.9 / 74.7 and
   // 79.5 / 76.5 / 71.3; FP16 16384^2, 16 warps of half the bytes, 106.9 / 107.8 /
-  // 107.9)
+  // 107.9; DRAM reads of a launch at 12288^2 on the first 11.8 GB at 32 rows, 12.5 at
+  // 64, the populations once 10.9)
   const int most = c->L.storage == 0 && c->L.P_bc == BC_PERIODIC && !c->L.force && P.smodel < 2
                        ? 32 : 64;
   const double slots = 152 * 15;
