@@ -55,7 +55,7 @@ def parse():
                          "divided into y-slabs, one per rank, halos exchanged every step")
     ap.add_argument("--instances", type=int, default=512)
     ap.add_argument("--schedule", default="auto", choices=["auto", "0", "1"],
-                    help="batch: launch schedule (0 persistent, 1 one launch per step; auto: "
+                    help="batch: launch schedule (0 persistent, 1 ordinary launches; auto: "
                          "the autotuner's choice over both)")
     ap.add_argument("--tiles", default="64x4", help="batch tile shape when --schedule is not auto")
     ap.add_argument("--boot", type=int, default=0,
@@ -253,40 +253,10 @@ def run_reference(args, world, rank):
 
 
 # ------------------------------------------------------------------ GPU arm
-def step_kernel(args):
-    """(name, time steps per launch) of the kernel that runs the Taylor-Green
-    context's steps for --step-path (unforced periodic n x n lattice; the rules of
-    run_step, choose_tile and march_min_nodes in csrc/ddflb_api.cu)."""
-    n, nodes, half = args.n, args.n * args.n, args.storage != "fp32"
-    plain = args.scalar_model in ("mrt", "srt")
-    if args.step_path == 0:
-        if -(-n // 32) * -(-n // 14) <= 152:
-            return "k_tile", 4
-        quad = half and plain and n % 4 == 0
-        two = (1.4e6 if not half else 1e7 if quad else 6e6) if plain else 1e7
-        if nodes >= two and (plain or not half):
-            return "k_march2", 2
-        if quad and nodes > 900000:
-            return "k_step_quad", 1
-        if nodes >= (85000 if not half else 0 if plain else 20000):
-            return "k_step_duo", 1
-        return "k_step", 1
-    if args.step_path == 3 and half and n % 4 == 0 and plain:
-        return "k_step_quad", 1
-    if args.step_path in (2, 3) and half and n % 2 == 0 and plain:
-        return "k_step_pair", 1
-    return "k_step", 1
-
-
-def step_kernel_name(args):
-    return step_kernel(args)[0]
-
-
-def traffic_per_launch(args, n_cells):
-    """DRAM bytes per step-kernel launch from the committed ncu summary, if it
-    was taken on the current kernel source (else None)."""
-    return traffic_record(f"{step_kernel_name(args)}_{args.storage}" + (
-        "" if args.scalar_model == "mrt" else f"_{args.scalar_model}"), n_cells)
+def traffic_key(kernel, args):
+    """The key of a step kernel's record in profiles/traffic.json."""
+    return f"{kernel}_{args.storage}" + ("" if args.scalar_model == "mrt"
+                                         else f"_{args.scalar_model}")
 
 
 def traffic_record(key, n_units):
@@ -385,7 +355,7 @@ def run_ours(args, world, rank, local):
         step_ms = sum(a.elapsed_time(b) for a, b, _ in ev)
         total_ms = max_over_ranks(world, total_ms)
         # lb steps take lb // T launches of T steps and single ones for the rest; then fields
-        T_launch = step_kernel(args)[1]
+        kernel, T_launch = lat.step_kernel()
         launches = args.steps * (lb // T_launch + lb % T_launch + 1)
 
         cells = n * n
@@ -444,12 +414,10 @@ def run_ours(args, world, rank, local):
                    "hbm_pct": round(100 * achieved / peak, 1)},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "peak_kind": kind,
-                     "kernel": step_kernel_name(args), "steps_per_launch": T_launch,
+                     "kernel": kernel, "steps_per_launch": T_launch,
                      "algorithmic_bytes_per_launch": algo_bytes,
-                     "traffic": traffic_per_launch(args, cells),
-                     "traffic_source": traffic_source(step_kernel_name(args) + "_" + args.storage
-                                                      + ("" if args.scalar_model == "mrt"
-                                                         else "_" + args.scalar_model),
+                     "traffic": traffic_record(traffic_key(kernel, args), cells),
+                     "traffic_source": traffic_source(traffic_key(kernel, args),
                                                       "cells of this launch")},
         "cpu_baseline": cpu,
         "e2e": e2e,
@@ -461,15 +429,15 @@ def run_ours(args, world, rank, local):
     print(json.dumps(line))
 
 
-def batch_launches(t0, lb, K=100):
+def batch_launches(t0, lb, per_launch, K=100):
     """(launches, passes over the populations) of one chunk of lb steps from step t0
-    under schedule 1: two steps per launch between the checks (every K steps),
-    single ones around them, with the sums and the check kernel after a check
+    under schedule 1: per_launch (two or one) steps per launch between the checks
+    (every K steps), single ones around them, with the sums and the check kernel after a check
     step, then the state-time update."""
     n, passes, k = 1, 0, 0
     while k < lb:
         t = t0 + k
-        two = k + 1 < lb and t % K and (t + 1) % K
+        two = per_launch == 2 and k + 1 < lb and t % K and (t + 1) % K
         n += 1 if t % K else 2 if t == 0 else 3
         passes += 1
         k += 2 if two else 1
@@ -550,8 +518,9 @@ def run_batch(args, world, rank, local):
         # this rank's kernel against this GPU's copy peak
         # every pass reads and writes the populations once (schedule 1: mostly two
         # steps per pass)
-        chunks = [batch_launches((args.warmup + k) * lb, lb) if tune["choice"][3] else (1, lb)
-                  for k in range(args.steps)]
+        per_launch = b.steps_per_launch()
+        chunks = [batch_launches((args.warmup + k) * lb, lb, per_launch) if tune["choice"][3]
+                  else (1, lb) for k in range(args.steps)]
         passes = sum(c[1] for c in chunks)
         achieved = 144 * cells * passes / (local_ms / 1e3) / 1e9
         # per-instance flags of the whole job, in global order, on rank 0
@@ -590,7 +559,8 @@ def run_batch(args, world, rank, local):
                    "l2": f"{288 * cells / 1e9:.1f} GB of populations on rank 0"},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "peak_kind": kind,
-                     "kernel": "k_batch" if tune["choice"][3] == 0 else "k_batch_march",
+                     "kernel": ("k_batch" if tune["choice"][3] == 0 else
+                                "k_batch_march" if per_launch == 2 else "k_batch_tile"),
                      "algorithmic_bytes_per_chunk": 144 * cells * chunks[0][1],
                      # bytes per node-step of schedule 0 from a 64-cavity capture, times a
                      # chunk's node-steps (every node-step moves the same 18 planes)
@@ -879,10 +849,10 @@ def run_sweep(args, world, rank, local):
                 torch.cuda.synchronize(dev)
                 ms = max_over_ranks(world, e0.elapsed_time(e1))
                 diverged = lat.stats()["diverged"]
+                kernel, steps_per_launch = lat.step_kernel()
                 del lat
             torch.cuda.empty_cache()
             bpc = BYTES_PER_CELL[st]
-            kernel, steps_per_launch = step_kernel(a)
             gbs = bpc * n * n * lb / steps_per_launch / (ms / 1e3) / 1e9
             rows.append({"n": n, "storage": st, "kernel": kernel,
                          "steps_per_launch": steps_per_launch,

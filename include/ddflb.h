@@ -317,6 +317,10 @@ ddflb_status ddflb_set_block(ddflb_ctx* c, int32_t block_x, int32_t block_y);
  * one on rows of at most 32 columns).  All give bit-identical results; which is
  * faster depends on the shape, so the autotuner times them. */
 ddflb_status ddflb_set_path(ddflb_ctx* c, int32_t path);
+/* The kernel that takes the context's steps (a static string) and the steps per
+ * launch, as path, size, storage and force have it now; either may be NULL.  Steps
+ * that a call or a check leaves over go one per launch. */
+ddflb_status ddflb_step_kernel(ddflb_ctx* c, const char** name, int32_t* steps_per_launch);
 
 /* Spatially varying part of the body force (Sec. 2; e.g. the four-rolls mill
  * of Sec. 5.2): dev_field is a device array [2][ny][nx] of floats (F_x plane,
@@ -438,6 +442,9 @@ ddflb_status ddflb_batch_set_instance_run(ddflb_batch* b, int32_t i, double tol,
  * The autotuner tries both. */
 ddflb_status ddflb_batch_set_schedule(ddflb_batch* b, int32_t schedule);
 ddflb_status ddflb_batch_get_schedule(const ddflb_batch* b, int32_t* schedule);
+/* Steps that one launch takes between two checks: a whole chunk (schedule 0), two
+ * or one (schedule 1, by the batch's sizes). */
+ddflb_status ddflb_batch_steps_per_launch(const ddflb_batch* b, int32_t* steps);
 /* Tile shape (32x4, 64x2, 128x1, 32x8, 64x4, 128x2, 256x1) and CTAs per SM
  * (0 = as many as fit); rebuilds the tile list.  Used by the autotuner. */
 ddflb_status ddflb_batch_set_tiles(ddflb_batch* b, int32_t tile_x, int32_t tile_y,

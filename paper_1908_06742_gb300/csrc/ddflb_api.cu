@@ -272,35 +272,46 @@ bool quad_pays(const Launch& L, int64_t nodes) {
   return nodes >= 3000000 && (L.P_bc == BC_CHANNEL || L.P.nx >= 8192);
 }
 
-cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void* fout, void* gout) {
-  const bool whole = c->L.P.y0 == 0 && c->L.P.y1 == c->L.P.ny;
-  const int64_t nodes = (int64_t)c->L.P.nx * c->L.P.ny;
-  // steps alternate their direction where the two buffers do not fit L2 together
-  const bool down = 2 * c->lay.pops_bytes > (size_t)80 << 20 && fin == c->pops[1];
+// The kernel of a single step.
+enum class Single { one, pair, quad, duo };
+
+Single single_kernel(const ddflb_ctx* c) {
+  const Launch& L = c->L;
+  const bool automatic = c->path == 0, whole = L.P.y0 == 0 && L.P.y1 == L.P.ny;
+  const int64_t nodes = (int64_t)L.P.nx * L.P.ny;
   // the kernels with one block row per lattice row end at the largest grid; beyond it
   // blocks of several rows (ddflb_set_block) step the lattice.  (A row offset in
   // k_step_duo instead cost its other lattices up to 1 %: 1023 x 767 FP16 1940 ->
   // 1959 us per 200 steps.)
-  const bool tall = c->path == 0 && c->L.P.ny > kMaxGridY;
-  const bool narrow = c->path == 0 && whole && narrow_rows(c->L, nodes);
-  const bool quad = quad_step_eligible(c->L) && !tall && !narrow;
-  // two nodes per thread in packed arithmetic
-  if (c->path == 0 && whole && !tall && !narrow && nodes >= duo_min_nodes(c->L) &&
-      !(quad && quad_pays(c->L, nodes))) {
-    auto* launch = c->L.storage == 0   ? launch_step_duo_f32
-                   : c->L.storage == 1 ? launch_step_duo_f16
-                                       : launch_step_duo_bf16;
-    return launch(c->L, fin, gin, fout, gout, c->status, down);
-  }
+  const bool tall = automatic && L.P.ny > kMaxGridY;
+  const bool narrow = automatic && whole && narrow_rows(L, nodes);
+  const bool quad = quad_step_eligible(L) && !tall && !narrow;
+  if (automatic && whole && !tall && !narrow && nodes >= duo_min_nodes(L) &&
+      !(quad && quad_pays(L, nodes)))
+    return Single::duo;
   // 16-bit storage steps node groups by default (wider accesses; bit-identical)
-  if ((c->path == 3 || c->path == 0) && quad)
-    return launch_step_quad(c->L, fin, gin, fout, gout, c->status, c->path == 0 && down);
+  if ((c->path == 3 || automatic) && quad) return Single::quad;
   // (with walls the paired kernel is no faster than one node per thread)
   const bool pair = c->path == 2 || c->path == 3 ||
-                    (tall && c->L.storage != 0 && c->L.P_bc == BC_PERIODIC);
-  if (pair && pair_step_eligible(c->L))
-    return launch_step_pair(c->L, fin, gin, fout, gout, c->status);
-  return launch_step(c->L, fin, gin, fout, gout, c->status);
+                    (tall && L.storage != 0 && L.P_bc == BC_PERIODIC);
+  return pair && pair_step_eligible(L) ? Single::pair : Single::one;
+}
+
+cudaError_t run_step(const ddflb_ctx* c, const void* fin, const void* gin, void* fout, void* gout) {
+  // steps alternate their direction where the two buffers do not fit L2 together
+  const bool down = 2 * c->lay.pops_bytes > (size_t)80 << 20 && fin == c->pops[1];
+  switch (single_kernel(c)) {
+    case Single::duo: {
+      auto* launch = c->L.storage == 0   ? launch_step_duo_f32
+                     : c->L.storage == 1 ? launch_step_duo_f16
+                                         : launch_step_duo_bf16;
+      return launch(c->L, fin, gin, fout, gout, c->status, down);
+    }
+    case Single::quad:
+      return launch_step_quad(c->L, fin, gin, fout, gout, c->status, c->path == 0 && down);
+    case Single::pair: return launch_step_pair(c->L, fin, gin, fout, gout, c->status);
+    default: return launch_step(c->L, fin, gin, fout, gout, c->status);
+  }
 }
 
 // Smallest lattice that takes two steps per launch: below it strips of enough rows
@@ -395,6 +406,13 @@ int choose_tile(const ddflb_ctx* c) {
     if ((int64_t)((P.nx + tx - 1) / tx) * ((P.ny + ty - 1) / ty) <= 152) return k;
   }
   return -1;
+}
+
+// What the automatic path takes, once after the path, the block or the force changed.
+void choose(ddflb_ctx* c) {
+  if (c->march_rows >= 0) return;
+  c->march_rows = choose_march_rows(c);
+  c->tile = choose_tile(c);
 }
 
 // kTileSteps steps from buffer src into the other one.
@@ -690,10 +708,7 @@ ddflb_status ddflb_step(ddflb_ctx* c, int64_t n) {
                               "refreshed between steps");
   Range range("ddflb_step");
   const int K = c->p.check_every;
-  if (c->march_rows < 0) {
-    c->march_rows = choose_march_rows(c);
-    c->tile = choose_tile(c);
-  }
+  choose(c);
   const bool single = capturing(c->L.stream);  // one step per launch, no graph of our own
   while (n > 0) {
     if (!single && c->p.force_omega == 0.0 && !c->graph_failed) {
@@ -1054,6 +1069,18 @@ ddflb_status ddflb_autotune(ddflb_ctx* c, int32_t trial_steps, int32_t* block_x,
   if (block_x) *block_x = (int32_t)bestb.x;
   if (block_y) *block_y = (int32_t)bestb.y;
   if (ms_per_step) *ms_per_step = best / trial_steps;
+  return DDFLB_OK;
+}
+
+ddflb_status ddflb_step_kernel(ddflb_ctx* c, const char** name, int32_t* steps) {
+  if (!c) return fail(DDFLB_EINVAL, "NULL handle");
+  choose(c);
+  static const char* const single[] = {"k_step", "k_step_pair", "k_step_quad", "k_step_duo"};
+  if (name)
+    *name = c->march_rows > 0 ? "k_march2"
+            : c->tile >= 0    ? "k_tile"
+                              : single[(int)single_kernel(c)];
+  if (steps) *steps = c->march_rows > 0 ? 2 : c->tile >= 0 ? kTileSteps : 1;
   return DDFLB_OK;
 }
 

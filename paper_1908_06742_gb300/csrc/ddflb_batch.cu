@@ -1018,6 +1018,12 @@ ddflb_status ddflb_batch_get_schedule(const ddflb_batch* b, int32_t* schedule) {
   return DDFLB_OK;
 }
 
+ddflb_status ddflb_batch_steps_per_launch(const ddflb_batch* b, int32_t* steps) {
+  if (!b || !steps) return bfail(DDFLB_EINVAL, "NULL argument");
+  *steps = b->schedule == 0 ? b->chunk : b->lay.two_steps ? 2 : 1;
+  return DDFLB_OK;
+}
+
 ddflb_status ddflb_batch_set_tiles(ddflb_batch* b, int32_t tile_x, int32_t tile_y,
                                    int32_t blocks_per_sm) {
   if (!b) return bfail(DDFLB_EINVAL, "NULL batch");

@@ -132,6 +132,9 @@ SIGNATURES = {
     "ddflb_nn_conv3x3_wgrad": (ctypes.c_int, [_FP] + [ctypes.c_int32] * 5 +
                                [_FP, ctypes.c_int32, ctypes.c_int32, _FP, ctypes.c_int32, _FP,
                                 _VP]),
+    "ddflb_step_kernel": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_char_p),
+                                         ctypes.POINTER(ctypes.c_int32)]),
+    "ddflb_batch_steps_per_launch": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_int32)]),
     "ddflb_nn_conv3x3_takes": (ctypes.c_int32, [ctypes.c_int32] * 6),
     "ddflb_nn_set_conv_path": (ctypes.c_int, [ctypes.c_int32]),
     "ddflb_nn_conv3x3_flip": (ctypes.c_int, [_FP, ctypes.c_int32, ctypes.c_int32, _FP, _VP]),
@@ -455,6 +458,12 @@ class Lattice:
         _check(self.lib.ddflb_set_path(self._h, int(path)))
         return self
 
+    def step_kernel(self):
+        """(name, steps per launch) of the kernel that takes this lattice's steps."""
+        name, steps = ctypes.c_char_p(), ctypes.c_int32()
+        _check(self.lib.ddflb_step_kernel(self._h, ctypes.byref(name), ctypes.byref(steps)))
+        return name.value.decode(), steps.value
+
     def state_bytes(self) -> int:
         return self.lib.ddflb_state_bytes(self._h)
 
@@ -596,6 +605,12 @@ class Batch:
     def schedule(self) -> int:
         v = ctypes.c_int32()
         _check(self.lib.ddflb_batch_get_schedule(self._h, ctypes.byref(v)))
+        return v.value
+
+    def steps_per_launch(self) -> int:
+        """Steps of one launch between two checks: the chunk (schedule 0), two or one."""
+        v = ctypes.c_int32()
+        _check(self.lib.ddflb_batch_steps_per_launch(self._h, ctypes.byref(v)))
         return v.value
 
     def set_instance_run(self, i, tol=-1.0, max_steps=0):
