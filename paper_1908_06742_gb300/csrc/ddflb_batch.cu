@@ -461,10 +461,9 @@ __global__ void __launch_bounds__(32, kMarchWarps<S, BC>)
   __syncwarp();
   const S* fin = (const S*)sI.buf[src];
   S* fout = (S*)sI.buf[src ^ 1];
-  if (!march_strip<S, BC>(sI.P, sK, fin, fin + sI.goff, fout, fout + sI.goff, T.y, T.z, T.w,
-                          march_shared, s_bar, s_wall) &&
-      threadIdx.x == 0)
-    atomicOr(&A.ist[T.x].flags, DDFLB_INST_LOST);  // no step, sum or check of it follows
+  march_strip<S, BC>(sI.P, sK, fin, fin + sI.goff, fout, fout + sI.goff, T.y, T.z, T.w,
+                     march_shared, s_bar, s_wall, &A.ist[T.x].flags,
+                     DDFLB_INST_LOST);  // (no step, sum or check of a lost instance follows)
 }
 
 __global__ void k_batch_advance(BatchSync* sync, int nsteps) {

@@ -113,14 +113,15 @@ constexpr size_t march_smem(int bc) {
 // cascaded 703 -> 605, central moments 691 -> 524).
 //
 // `strip` and rows [y0, y1) name the strip and chunk; shared: march_smem() bytes;
-// bars: STAGES mbarriers; wall: 12 floats.  False if a copy did not arrive (the rest of
-// the chunk is then not written).
+// bars: STAGES mbarriers; wall: 12 floats.  If a copy does not arrive, the rest of the
+// chunk is not written and *stop, 0 until then, takes `bit` (a plain store: the same
+// from every warp; an atomic cost the cavity forms registers).
 template <typename S, int BC, bool FORCE = false, int SM = 0>
-__device__ __forceinline__ bool march_strip(const LbParams& P, const PairConst& K,
+__device__ __forceinline__ void march_strip(const LbParams& P, const PairConst& K,
                                             const S* __restrict__ fin, const S* __restrict__ gin,
                                             S* __restrict__ fout, S* __restrict__ gout, int strip,
                                             int y0, int y1, unsigned char* shared, uint64_t* bars,
-                                            float* s_wall) {
+                                            float* s_wall, int* stop, int bit) {
   using Io = PairIo<S>;
   constexpr bool COMP = sizeof(S) == 4;
   static_assert(COMP || !(FORCE || SM), "16-bit storage: unforced MRT only");
@@ -418,7 +419,7 @@ __device__ __forceinline__ bool march_strip(const LbParams& P, const PairConst& 
     up1 = t;
   }
   if (bad) {
-    // a copy did not arrive: let those in flight land (bounded)
+    // a copy did not arrive: let those in flight land (bounded), then report
     for (int k = 0; k < NST; ++k) {
       phase_wait(bar0 + 8 * st, phase);
       if (++st == NST) {
@@ -426,8 +427,8 @@ __device__ __forceinline__ bool march_strip(const LbParams& P, const PairConst& 
         phase ^= 1;
       }
     }
+    if (lane == 0) *stop = bit;
   }
-  return !bad;
 }
 
 template <typename S, int BC, bool FORCE, int SM>
@@ -440,10 +441,8 @@ __global__ void __launch_bounds__(32, kMarchWarps<S, BC, FORCE, SM>)
   __shared__ float s_wall[12];  // cavity: the side walls' links in row i
   if (status->stopped) return;
   const int y0 = blockIdx.y * rows;
-  if (!march_strip<S, BC, FORCE, SM>(P, K, fin, gin, fout, gout, blockIdx.x, y0,
-                                     min(y0 + rows, P.ny), march_shared, s_bar, s_wall) &&
-      threadIdx.x == 0)
-    atomicOr(&status->stopped, kStopTimeout);
+  march_strip<S, BC, FORCE, SM>(P, K, fin, gin, fout, gout, blockIdx.x, y0, min(y0 + rows, P.ny),
+                                march_shared, s_bar, s_wall, &status->stopped, kStopTimeout);
 }
 
 namespace march {
